@@ -274,11 +274,14 @@ int wsfft_plan_set_ragged_variant(wsfft_plan plan, int shape_select, int lag);
  * in split form (real parts together, imaginary parts together) so that its
  * butterflies run as packed FP32x2 instructions; tile code 2000 selects the
  * tensor-core contiguous superstep (16-bit storage, N = 512; the
- * values-per-thread argument is then ignored).  Used by the autotuner.
+ * values-per-thread argument is then ignored); tile codes 4013 and 4014
+ * select the pipelined strided kernel with 2^13 or 2^14 elements per tile
+ * (values per thread: the radix of its first stage, 8 up to 64 points, 16 up
+ * to 256, 32 above).  Used by the autotuner.
  * Errors: INVALID_ARG, UNSUPPORTED (that shape is not built for this pass).
- * A shape that needs whole tiles (either pencil-pair kernel) on a pass whose
- * pencil count or stride is not a multiple of its tile makes wsfft_execute
- * return CUDA without launching. */
+ * A shape that needs whole tiles (either pencil-pair kernel, the pipelined
+ * kernel) on a pass whose pencil count or stride is not a multiple of its
+ * tile makes wsfft_execute return UNSUPPORTED without launching. */
 int wsfft_plan_set_pass_variant(wsfft_plan plan, int pass, int values_per_thread, int tile);
 
 /* Choose the schedule of a rank-3 transform n0 x n x n (n in {128, 256, 512,

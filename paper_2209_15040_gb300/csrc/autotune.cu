@@ -149,8 +149,15 @@ double time_plan(Plan &p, const void *in, void *out, cudaStream_t st) {
     return ok && ms >= 0.f ? ms * 1e3 / 3.0 : -1.0;
 }
 
-// (kind, N, storage type) -> extra shapes instantiated by pass_launch.cuh
+// (kind, N, storage type) -> extra shapes instantiated by pass_launch.cuh and
+// tile_launch.cuh (a tile of 0 pencils: the general shape of that length)
 std::vector<std::pair<int, int>> shapes_for(int kind, int N, int dtype) {
+    if (kind == PASS_STRIDED && dtype != WSFFT_C32) {
+        if (N == 32 || N == 64) return {{8, 0}, {8, PIPE_TILE + 13}};
+        if (N == 128) return {{16, 0}, {16, PIPE_TILE + 13}};
+        if (N == 256)
+            return {{16, 0}, {16, 32}, {8, 16}, {8, PAIR_TILE + 16}, {16, PIPE_TILE + 13}, {16, PIPE_TILE + 14}};
+    }
     // tensor-core DFT-16 stage (16-bit storage only)
     if (kind == PASS_CONTIG && N == 512 && dtype != WSFFT_C32)
         return {{32, 16}, {32, 8}, {32, 32}, {16, 8}, {8, 8}, {16, TC_TILE}, {16, SPLIT_TILE + 8},
@@ -158,9 +165,10 @@ std::vector<std::pair<int, int>> shapes_for(int kind, int N, int dtype) {
     if (kind == PASS_STRIDED && N == 512)
         return {{32, 16}, {32, 8},  {32, 32}, {16, 16}, {8, 8}, {16, 8}, {16, 32}, {8, PAIR_TILE + 16},
                 {8, PAIR_TILE + 32}, {8, PAIR_TILE + 8}, {16, PAIR_TILE + 16}, {16, PAIR_TILE + 32},
-                {16, SPLIT_TILE + 16}, {16, SPLIT_TILE + 32}, {8, SPLIT_TILE + 16}, {8, SPLIT_TILE + 32}};
+                {16, SPLIT_TILE + 16}, {16, SPLIT_TILE + 32}, {8, SPLIT_TILE + 16}, {8, SPLIT_TILE + 32},
+                {32, PIPE_TILE + 13}, {32, PIPE_TILE + 14}};
     if (kind == PASS_STRIDED && N == 256) return {{16, 32}, {8, 16}, {8, PAIR_TILE + 16}};
-    if (kind == PASS_STRIDED && N == 1024) return {{16, 8}, {32, 8}, {16, SPLIT_TILE + 8}};
+    if (kind == PASS_STRIDED && N == 1024) return {{16, 8}, {32, 8}, {32, 16}, {16, SPLIT_TILE + 8}, {32, PIPE_TILE + 14}};
     if (kind == PASS_CONTIG && N == 512)
         return {{32, 16}, {32, 8}, {32, 32}, {16, 8}, {8, 8}, {16, SPLIT_TILE + 8}, {16, SPLIT_TILE + 16}};
     if (kind == PASS_CONTIG && N == 256) return {{8, 8}};

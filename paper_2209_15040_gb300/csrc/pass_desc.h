@@ -45,6 +45,8 @@ struct PassArgs {
     int *status;        // plan's device status word (kernels with bounded waits)
     uint64_t timeout_ns;  // bound of each wait
     int reverse;        // strided launches: 1 = blocks take the tiles from the last one down
+    // pipelined tiles (tile.cuh)
+    int64_t tiles;      // tiles of the launch
 };
 
 // tile codes at or above this select the complex64 pencil-pair strided
@@ -61,6 +63,9 @@ constexpr int TC_TABLE_FLOAT2 = 768;
 // tile codes at or above this select the split-form pencil-pair strided
 // kernel (packed FP32x2 butterflies) with (code - SPLIT_TILE) pencils per block
 constexpr int SPLIT_TILE = 3000;
+// tile codes at or above this select the pipelined tile kernels (tile.cuh)
+// with 2^(code - PIPE_TILE) elements per tile
+constexpr int PIPE_TILE = 4000;
 
 enum PassKind {
     PASS_CONTIG = 0,     // one launch, contiguous axis

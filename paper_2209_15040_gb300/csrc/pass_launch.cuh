@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "launch_util.h"
 #include "pass_kernels.cuh"
 #include "tc_contig.cuh"
 
@@ -22,28 +23,8 @@ cudaError_t set_smem(K kernel, int bytes) {
 
 inline bool plain_pass(const PassArgs &a) { return a.conj_in == 1.f && a.sx == 1.f && a.sy == 1.f; }
 
-// Launch with programmatic stream serialization (see pdl_enter): the kernel
-// may begin launching while the previous kernel in the stream drains.  Used
-// for passes over at most 2 GiB: measured 0.7% faster per transform at 512^3
-// and 5% at 256^3, but 14% slower at 1024^3 (8 GiB), so larger passes
-// launch plainly.
 inline bool pdl_pass(const PassArgs &a, int N, int elem_bytes) {
-    return a.npencils * (int64_t)N * elem_bytes <= ((int64_t)2 << 30);
-}
-template <class... KArgs, class... Args>
-cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), unsigned grid, unsigned block, int smem,
-                       cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    return pdl_bytes(a.npencils * (int64_t)N * elem_bytes);
 }
 
 template <int N, int E, int P, class S, bool TRANS>

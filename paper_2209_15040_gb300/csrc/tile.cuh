@@ -1,0 +1,359 @@
+// Pipelined supersteps over tiles of 2^13 or 2^14 elements.
+//
+// Persistent blocks transform one tile in registers while asynchronous copies
+// bring the next tile's elements into shared memory, so the loads of tile
+// i+1 run under the last stage and the stores of tile i.
+//
+// The TB bits of an element's index in the tile are its "slots".  In every
+// stage a thread holds 64 elements: five slots index its registers (the
+// digits the stage transforms, plus spare slots when they are shorter), one
+// slot is the pair of elements that share packed FP32x2 instructions (cpair),
+// and the others are the thread index.  A stage replaces a digit's slots
+// by the digit of frequency with the same bits, so between stages only the
+// roles of the slots change: an exchange writes each value to the
+// shared-memory address of its slots and reads the values of the next
+// stage's.  Addresses are linear in the bits, so each is one per-thread base
+// plus a compile-time offset.
+//
+// Tiles of 2^13 elements: 128 threads, two blocks per SM in complex64, three
+// in 16-bit storage.  The exchanges run through the load buffer, which takes
+// the next tile once the last exchange has been read; the blocks of an SM
+// are in different phases, so one's arithmetic runs under another's shared
+// memory traffic.  Tiles of 2^14 elements (256 threads, one block per SM) are
+// for axes whose rows would fall below 128 bytes otherwise: they have a load
+// buffer of their own (128 KB in complex64), and real and imaginary parts
+// pass through a 70 KB exchange buffer one after the other.
+#pragma once
+
+#include "pass_kernels.cuh"
+#include "tile_desc.h"
+
+namespace wsfft {
+
+__device__ __forceinline__ void cp_async16(void *smem, const void *g) {
+    const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(g) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// ---------------------------------------------------------------------------
+// Geometries: which slots each stage transforms.  A geometry G has
+//   NST                stages
+//   pair(s)            slot of the pair
+//   in(s, j)           slot of register bit j (the digit first, then spares)
+//   gbits(s)           bits of the digit
+//   nsbits(s), kslot(s, i)  bits of the frequency so far (0: no twiddle) and
+//                      the slot of its bit i
+//   ls(slot), LBUF     load-buffer stride of a slot, elements of the buffer
+
+// Slots of a tile of 2^NB points x 2^(TB-NB) pencils: pencil bits first, then
+// the axis.  Two stages: the high R0 bits of the axis, then the low R1 bits.
+template <int TBITS, int NB>
+struct TileAxis {
+    static_assert(NB >= 5 && NB <= 10, "two register stages");
+    static constexpr int LW = TBITS - NB, W = 1 << LW, N = 1 << NB;
+    static constexpr int R0 = NB >= 9 ? 5 : NB >= 7 ? 4 : 3, R1 = NB - R0;
+    static constexpr int TB = TBITS;
+    static constexpr int NST = 2;
+    __host__ __device__ static constexpr int gbits(int s) { return s == 0 ? R0 : R1; }
+    __host__ __device__ static constexpr int nsbits(int s) { return s == 0 ? 0 : R0; }
+    __host__ __device__ static constexpr int kslot(int, int i) { return TBITS - R0 + i; }
+    __host__ __device__ static constexpr int in(int s, int j) {
+        if (j < gbits(s)) return (s == 0 ? TBITS - R0 : LW) + j;
+        // spares: the top pencil bits (a pencil's exchange then stays in fewer
+        // threads); 512 points: the top frequency bit
+        return NB <= 8 ? LW - 1 - (j - gbits(s)) : TBITS - 1;
+    }
+    static constexpr int TABLE = ((1 << R1) - 1) << R0;  // entries of the twiddle table
+};
+
+// Strided axis: 2^LW adjacent pencils, rows of the tile copied whole.
+template <int TBITS, int NB>
+struct TileStrided : TileAxis<TBITS, NB> {
+    static constexpr int LBUF = (1 << TBITS);
+    static constexpr int ROWBITS = TileAxis<TBITS, NB>::LW, XROWS = 1 << NB;  // elements per row, rows
+    __host__ __device__ static constexpr int pair(int) { return 0; }
+    __host__ __device__ static constexpr int ls(int slot) { return 1 << slot; }
+};
+
+// Slot j of the thread index: the slots that are neither in a register nor
+// the pair, lowest first.
+template <class G>
+__host__ __device__ constexpr int tile_th(int s, int j) {
+    int c = 0;
+    for (int slot = 0; slot < G::TB; ++slot) {
+        bool used = slot == G::pair(s);
+        for (int i = 0; i < 5; ++i) used |= G::in(s, i) == slot;
+        if (used) continue;
+        if (c == j) return slot;
+        ++c;
+    }
+    return -1;
+}
+
+// Exchange layout after stage E: the stride (floats) of a slot.  Slots take
+// positions (powers of two): the pair first where both stages have the same
+// one (it moves as 8 bytes), the writing stage's lanes next - those that are
+// also lanes of the reading stage first -, then the slots that are no lanes,
+// and on top the reading stage's other lanes, `nr` of them.  A pad of
+// 2^(5-nr) floats per step of the lowest of these gives them the banks of the
+// writing stage's other lanes: writes and reads are free of bank conflicts.
+template <class G>
+__host__ __device__ constexpr int tile_xs(int e, int slot) {
+    const bool vec = G::pair(e) == G::pair(e + 1);
+    const int lanes = vec ? 4 : 5;  // lanes that share one pass of the banks
+    int order[16] = {};
+    bool placed[16] = {};
+    int c = 0, nr = 0;
+    if (vec) {
+        order[c++] = G::pair(e);
+        placed[G::pair(e)] = true;
+    }
+    for (int both = 1; both >= 0; --both)
+        for (int j = 0; j < lanes; ++j) {
+            const int t = tile_th<G>(e, j);
+            bool in_r = false;
+            for (int i = 0; i < lanes; ++i) in_r |= tile_th<G>(e + 1, i) == t;
+            if (in_r == (both == 1)) {
+                order[c++] = t;
+                placed[t] = true;
+            }
+        }
+    for (int j = 0; j < lanes; ++j) nr += placed[tile_th<G>(e + 1, j)] ? 0 : 1;
+    for (int t = 0; t < G::TB; ++t) {
+        bool r_lane = false;
+        for (int j = 0; j < lanes; ++j) r_lane |= tile_th<G>(e + 1, j) == t;
+        if (!placed[t] && !r_lane) order[c++] = t;
+    }
+    for (int j = 0; j < lanes; ++j)
+        if (!placed[tile_th<G>(e + 1, j)]) order[c++] = tile_th<G>(e + 1, j);
+    for (int i = 0; i < G::TB; ++i)
+        if (order[i] == slot) return (1 << i) + (i >= G::TB - nr ? 1 << (i - (G::TB - nr) + 5 - nr) : 0);
+    return -1;
+}
+template <class G>
+__host__ __device__ constexpr int tile_xfloats() {
+    int most = 0;
+    for (int e = 0; e + 1 < G::NST; ++e) {
+        int n = 1;
+        for (int t = 0; t < G::TB; ++t) n += tile_xs<G>(e, t);
+        most = n > most ? n : most;
+    }
+    return (most + 3) & ~3;
+}
+
+// Kinds of address: load buffer, exchange after stage E, slot number.
+enum { TILE_OFF_LOAD = -2, TILE_OFF_SLOT = -1 };
+template <class G, int KIND>
+__host__ __device__ constexpr int tile_stride(int slot) {
+    return KIND == TILE_OFF_LOAD ? G::ls(slot) : KIND == TILE_OFF_SLOT ? 1 << slot : tile_xs<G>(KIND, slot);
+}
+template <class G, int KIND, int SG, int J = 0>
+__device__ __forceinline__ int tile_thread_off(int tid) {
+    if constexpr (J == G::TB - 6) {
+        return 0;
+    } else {
+        constexpr int st = tile_stride<G, KIND>(tile_th<G>(SG, J));
+        return ((tid >> J) & 1) * st + tile_thread_off<G, KIND, SG, J + 1>(tid);
+    }
+}
+template <class G, int KIND, int SG>
+__host__ __device__ constexpr int tile_reg_off(int r) {
+    int o = 0;
+    for (int j = 0; j < 5; ++j)
+        if ((r >> j) & 1) o += tile_stride<G, KIND>(G::in(SG, j));
+    return o;
+}
+// frequency so far that a set of slots holds
+template <class G, int SG>
+__host__ __device__ constexpr int tile_k_of(int slots) {
+    int k = 0;
+    for (int i = 0; i < G::nsbits(SG); ++i) k |= ((slots >> G::kslot(SG, i)) & 1) << i;
+    return k;
+}
+
+// Read one part (real or imaginary) of a stage's values, or write it.
+template <class G, int E, int SG, bool IM, bool WRITE, int R = 0>
+__device__ __forceinline__ void tile_part(cpair (&v)[32], float *x) {
+    if constexpr (R < 32) {
+        constexpr int PS = tile_xs<G>(E, G::pair(SG));
+        constexpr int off = tile_reg_off<G, E, SG>(R);
+        float2 &p = IM ? v[R].im : v[R].re;
+        if constexpr (PS == 1) {
+            if constexpr (WRITE) *reinterpret_cast<float2 *>(x + off) = p;
+            else p = *reinterpret_cast<const float2 *>(x + off);
+        } else if constexpr (WRITE) {
+            x[off] = p.x;
+            x[off + PS] = p.y;
+        } else {
+            p.x = x[off];
+            p.y = x[off + PS];
+        }
+        tile_part<G, E, SG, IM, WRITE, R + 1>(v, x);
+    }
+}
+// Exchange between stages E and E+1.  FULL: room for both parts at once (one
+// barrier); otherwise they take turns in one buffer.
+template <class G, int E, bool FULL>
+__device__ __forceinline__ void tile_exchange(cpair (&v)[32], float *xw, float *xr) {
+    constexpr int IM = FULL ? tile_xfloats<G>() : 0;
+    if constexpr (E > 0) __syncthreads();  // the previous exchange has been read
+    tile_part<G, E, E, false, true>(v, xw);
+    if constexpr (FULL) tile_part<G, E, E, true, true>(v, xw + IM);
+    __syncthreads();
+    tile_part<G, E, E + 1, false, false>(v, xr);
+    if constexpr (!FULL) {
+        __syncthreads();
+        tile_part<G, E, E, true, true>(v, xw);
+        __syncthreads();
+    }
+    tile_part<G, E, E + 1, true, false>(v, xr + IM);
+}
+
+// A stage: the digit's twiddles and its DFT.  The twiddles multiply all
+// values before the first butterfly (interleaved with the butterflies the
+// compiler's schedule was 10% slower).
+template <class G, int SG, bool LDG>
+__device__ __forceinline__ void tile_stage(cpair (&v)[32], const float2 *__restrict__ tw, int slots) {
+    constexpr int B = G::gbits(SG), R = 1 << B, NSB = G::nsbits(SG);
+    if constexpr (NSB > 0) {
+        const float2 *tk = tw + tile_k_of<G, SG>(slots);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const int r = i & (R - 1);
+            if (r == 0) continue;
+            const float2 *p = tk + (((r - 1) << NSB) + tile_k_of<G, SG>(tile_reg_off<G, TILE_OFF_SLOT, SG>(i)));
+            v[i] = cmul(v[i], LDG ? __ldg(p) : *p);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 32; i += R) {
+        cpair g[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) g[r] = v[i + r];
+        dft_fused<R>(g);
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[i + r] = g[r];
+    }
+}
+
+// Shared memory: load buffer, exchange buffer (the same bytes in tiles of
+// 2^13 elements), then (16-bit storage) the stage twiddles.
+template <class G, class S>
+struct TileSmem {
+    static constexpr int CTAS = G::TB == 14 ? 1 : sizeof(S) == 4 ? 3 : 2;  // blocks per SM
+    static constexpr bool SHARED_BUF = G::TB < 14;
+    // both parts of an exchange at once where there is room (16-bit tiles of
+    // 2^14: 2-4% faster)
+    static constexpr bool FULL = SHARED_BUF || sizeof(S) == 4;
+    static constexpr int LOAD = G::LBUF * (int)sizeof(S), XCHG = tile_xfloats<G>() * (FULL ? 8 : 4);
+    static constexpr int X = SHARED_BUF ? 0 : LOAD;
+    static constexpr int TW = SHARED_BUF ? (LOAD > XCHG ? LOAD : XCHG) : LOAD + XCHG;
+    // 16-bit storage is bound by the SM and reads its stage twiddles 5%
+    // faster from shared memory; complex64 is bound by HBM and was slower so
+    static constexpr bool SHARED_TW = sizeof(S) == 4;
+    static constexpr int BYTES = TW + (SHARED_TW ? G::TABLE * 8 : 0);
+    static_assert(BYTES <= 228 * 1024 / CTAS - 1024, "blocks per SM");
+};
+
+// Superstep along a strided axis.  What bounds it and what it gives, 2^27
+// elements, against the one-tile-per-block kernels of pass_kernels.cuh:
+//   complex64, 1024 points, 16 pencils (tiles of 2^14): the memory system, on
+//     128-byte rows (the same copies and stores without arithmetic take as
+//     long); 0.343 ms against 0.410 (8 pencils, 64-byte rows) and 0.49-0.51
+//     (16 pencils, one block per SM without the copies in flight) at a stride
+//     of 2^10, 0.39 against 0.46-0.50 at 2^17;
+//   16-bit storage: the SM -- FP32 pipe and shared memory, which the blocks
+//     of an SM overlap in part: 512 points 0.20 ms (tiles of 2^13), 0.227
+//     (2^14) against 0.26-0.27; 256 points 0.187 and 0.205 against 0.24-0.25.
+template <class G, class S>
+__global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S>::CTAS)
+    tile_strided_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
+    using SM = TileSmem<G, S>;
+    using PT = typename SplitPair<S>::T;
+    constexpr int NT = 1 << (G::TB - 6);
+    constexpr bool LDG = !SM::SHARED_TW;
+    extern __shared__ float4 t_smem[];
+    char *sm = reinterpret_cast<char *>(t_smem);
+    float *xb = reinterpret_cast<float *>(sm + SM::X);
+    const int tid = threadIdx.x;
+    const float2 *tw = a.tw;
+    if constexpr (SM::SHARED_TW) {
+        // a plan's table: no kernel writes it
+        float2 *st = reinterpret_cast<float2 *>(sm + SM::TW);
+        for (int i = tid; i < G::TABLE; i += NT) st[i] = a.tw[i];
+        tw = st;
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int64_t ntiles = a.tiles;
+
+    // first element of a tile
+    auto tile_base = [&](int64_t t) -> int64_t {
+        const int64_t q = (a.reverse ? ntiles - 1 - t : t) * G::W;
+        return ((q >> a.log_inner) * ((int64_t)G::N << a.log_inner)) + (q & (a.inner - 1));
+    };
+    auto issue = [&](int64_t tile) {
+        constexpr int EPC = 16 / (int)sizeof(S), CPR = G::W / EPC, ROWS = NT / CPR;  // chunks per row, rows per round
+        static_assert(CPR <= NT && G::N % ROWS == 0, "whole rounds");
+        const S *p = in + tile_base(tile) + (int64_t)(tid / CPR) * a.inner + (tid % CPR) * EPC;
+        const int64_t step = (int64_t)ROWS * a.inner;
+#pragma unroll
+        for (int j = 0; j < G::N / ROWS; ++j) {
+            cp_async16(sm + (tid + j * NT) * 16, p);
+            p += step;
+        }
+    };
+    // start the copies of the tile after `tile`
+    auto next = [&](int64_t tile) {
+        if (tile + gridDim.x < ntiles) issue(tile + gridDim.x);
+        else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        cp_async_commit();
+    };
+    const S *lbuf = reinterpret_cast<const S *>(sm) + tile_thread_off<G, TILE_OFF_LOAD, 0>(tid);
+    float *xw = xb + tile_thread_off<G, 0, 0>(tid), *xr = xb + tile_thread_off<G, 0, 1>(tid);
+    const int slots = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid);
+    const int wcol = slots & (G::W - 1), k1 = tile_k_of<G, 1>(slots);
+
+    int64_t tile = blockIdx.x;
+    if (tile < ntiles) issue(tile);
+    cp_async_commit();
+    for (; tile < ntiles; tile += gridDim.x) {
+        cpair v[32];
+        cp_async_wait_all();
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+            v[r] = SplitPair<S>::load(reinterpret_cast<const PT *>(lbuf + tile_reg_off<G, TILE_OFF_LOAD, 0>(r)));
+            v[r].im = __fmul2_rn(v[r].im, f2dup(a.conj_in));
+        }
+        __syncthreads();
+        if constexpr (!SM::SHARED_BUF) next(tile);
+        tile_stage<G, 0, LDG>(v, tw, 0);
+        tile_exchange<G, 0, SM::FULL>(v, xw, xr);
+        if constexpr (SM::SHARED_BUF) {
+            __syncthreads();
+            next(tile);
+        }
+        tile_stage<G, 1, LDG>(v, tw, slots);
+        // row k = k1 + Ns k2: k2 in the registers
+        constexpr int Ns = 1 << G::R0, R = 1 << G::R1;
+        S *o = out + tile_base(tile) + (int64_t)k1 * a.inner + wcol;
+        const int64_t step = (int64_t)Ns * a.inner;
+#pragma unroll
+        for (int i = 0; i < 32; i += R) {
+            const int sp = tile_reg_off<G, TILE_OFF_SLOT, 1>(i);
+            S *p = o + (int64_t)tile_k_of<G, 1>(sp) * a.inner + (sp & (G::W - 1));
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                cpair z = v[i + r];
+                z.re = __fmul2_rn(z.re, f2dup(a.sx));
+                z.im = __fmul2_rn(z.im, f2dup(a.sy));
+                SplitPair<S>::store(reinterpret_cast<PT *>(p), z);
+                p += step;
+            }
+        }
+    }
+}
+
+}  // namespace wsfft

@@ -1,0 +1,21 @@
+// Host-visible interface of the pipelined tile kernels (tile.cuh).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "pass_desc.h"
+
+namespace wsfft {
+
+// Values per thread of the twiddle table a tile kernel's axis of length N
+// uses: the radix of its first stage.
+inline int tile_table_E(int N) { return N <= 64 ? 8 : N <= 256 ? 16 : 32; }
+
+// Launch one superstep along a strided axis on the pipelined tile kernels.
+// tb: log2 of the elements per tile.  Returns cudaErrorInvalidValue
+// for a shape that is not instantiated or does not divide into whole tiles.
+cudaError_t launch_tile_c32(int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_c16f(int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_c16bf(int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+
+}  // namespace wsfft

@@ -38,6 +38,7 @@
 #include "ragged_desc.h"
 #include "slab_cluster.cuh"
 #include "slab_desc.h"
+#include "tile_desc.h"
 
 namespace wsfft {
 
@@ -187,8 +188,21 @@ cudaError_t launch_slab(int dtype, int n, const void *in, void *out, int64_t nsl
     }
 }
 
+cudaError_t launch_tile(int dtype, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st) {
+    switch (dtype) {
+        case WSFFT_C32: return launch_tile_c32(N, tb, in, out, a, st);
+        case WSFFT_C16F: return launch_tile_c16f(N, tb, in, out, a, st);
+        default: return launch_tile_c16bf(N, tb, in, out, a, st);
+    }
+}
+
 cudaError_t launch(int dtype, const PassSpec &p, const void *in, void *out, const PassArgs &a,
                    cudaStream_t st) {
+    if (p.tile >= PIPE_TILE) {
+        // the kernels' stage tables are those of one radix per axis length
+        if (p.kind != PASS_STRIDED || p.variant || p.E != tile_table_E(p.N)) return cudaErrorInvalidValue;
+        return launch_tile(dtype, p.N, p.tile - PIPE_TILE, in, out, a, st);
+    }
     switch (dtype) {
         case WSFFT_C32: return launch_pass_c32(p.kind, p.N, p.E, p.tile, p.variant, in, out, a, st);
         case WSFFT_C16F: return launch_pass_c16f(p.kind, p.N, p.E, p.tile, p.variant, in, out, a, st);
@@ -204,6 +218,32 @@ int cuda_status(cudaError_t e) { return e == cudaSuccess ? WSFFT_SUCCESS : WSFFT
 // checked separately (Plan::overrides_launchable)
 bool override_usable(int E, int tile, int N) {
     return E >= 1 && E <= 32 && E <= N && (E & (E - 1)) == 0 && tile >= 0;
+}
+
+// log2 of the elements per tile with which a strided superstep of length N at
+// element stride `inner`, over `total` elements, runs on the pipelined tile
+// kernels; 0: the one-tile-per-block kernels are faster, or the pencils do
+// not fill whole tiles.  Measured per superstep, against those kernels:
+//   complex64: 1024 points from 2^25 elements up (2^25 102-107 us against
+//     99-108, 2^27 351-383 against 374-501; 2^23 26.0 against 23.9: too few
+//     tiles of 128 KB per SM); shorter axes are at the copy rate without them.
+//   16-bit storage: from 2^22 elements up (2^27 170-174 us against 224-273
+//     at 32..128 points, 185-206 against 235-251 at 256, 200-212 against
+//     255-271 at 512, 234-237 against 330-338 at 1024; within 0.5 us of each
+//     other below).  Tiles of 2^13 elements (three blocks per SM) are the
+//     faster ones until their rows (64 bytes at 512 points, 128 at 256, 256 at
+//     128) lie 2^19 to 2^22 bytes apart: 512 points 206 us at a stride of
+//     2^16 elements and 282 at 2^18, where tiles of 2^14 take 210 and 212.
+int pipe_tile_bits(int dtype, int64_t N, int64_t inner, int64_t total) {
+    int tb = 0;
+    if (dtype == WSFFT_C32) {
+        if (N == 1024 && total >= ((int64_t)1 << 25)) tb = 14;
+    } else if (total >= ((int64_t)1 << 22)) {
+        if (N == 32 || N == 64 || N == 128) tb = inner <= ((int64_t)1 << 18) ? 13 : 0;
+        if (N == 256 || N == 512) tb = inner < ((int64_t)1 << 17) ? 13 : 14;
+        if (N == 1024) tb = 14;
+    }
+    return tb && inner % (((int64_t)1 << tb) / N) == 0 ? tb : 0;
 }
 
 // two buffers of `bytes` that share some bytes without being the same buffer
@@ -535,6 +575,14 @@ int Plan::build_schedule() {
             if (dtype == WSFFT_C32 && inner >= ((int64_t)1 << 17)) {
                 p.E = 32;
                 p.tile = 16;
+            }
+        }
+        if (p.kind == PASS_STRIDED) {
+            // pipelined tile kernels (tile.cuh) where whole tiles fit
+            const int tb = pipe_tile_bits(dtype, p.N, inner, elems * batch);
+            if (tb) {
+                p.E = tile_table_E(p.N);
+                p.tile = PIPE_TILE + tb;
             }
         }
     };

@@ -1,0 +1,76 @@
+"""GPU parity of the pipelined tile kernels (csrc/tile.cuh): every instantiated
+shape at the smallest stride it takes, with fewer tiles than resident blocks,
+one tile, and a last round that only some blocks take; both directions; in
+place; and the plan builder's rule against the general kernels on strides on
+both sides of its limits.  Tolerances are those of the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2209_15040_gb300 import build
+from paper_2209_15040_gb300 import wsfft as W
+from tests._helpers import DT, TOL, seeded, to_device, to_host_c128
+
+pytestmark = pytest.mark.gpu
+
+PIPE = 4000
+# (points, values per thread, log2 elements per tile)
+HALF = [(32, 8, 13), (64, 8, 13), (128, 16, 13), (256, 16, 13), (256, 16, 14), (512, 32, 13), (512, 32, 14),
+        (1024, 32, 14)]
+SHAPES = [(d, *s) for d in ("c16f", "c16bf") for s in HALF] + [("c32", 1024, 32, 14)]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build_library()
+    W.lib()
+    torch.cuda.init()
+
+
+def _axis(x, dtype, n, inner, batch, direction, variant):
+    plan = W.AxisPlan(n, inner, DT[dtype], direction, batch, norm=W.NORM_ORTHO)
+    try:
+        if variant:
+            plan.set_pass_variant(0, *variant)
+        out = torch.empty_like(x)
+        plan.execute(x.data_ptr(), out.data_ptr())
+        same = x.clone()
+        plan.execute(same.data_ptr(), same.data_ptr())
+        torch.cuda.synchronize()
+    finally:
+        plan.close()
+    assert torch.equal(out, same)  # in place: the same bytes
+    return out
+
+
+@pytest.mark.parametrize("dtype,n,e,tb", SHAPES)
+@pytest.mark.parametrize("tiles", ["one", "few", "rounds"])
+def test_strided_tile_shapes(dtype, n, e, tb, tiles):
+    w = (1 << tb) // n
+    inner = w if tiles == "one" else 2 * w
+    blocks = torch.cuda.get_device_properties(0).multi_processor_count * (1 if tb == 14 else 3)
+    batch = {"one": 1, "few": 5, "rounds": blocks // 2 + 3}[tiles]
+    direction = W.INVERSE if tiles == "few" else W.FORWARD
+    xs, xc = seeded((batch, n, inner), 11, "uniform", dtype)
+    got = to_host_c128(_axis(to_device(xs, dtype), dtype, n, inner, batch, direction, (e, PIPE + tb)), dtype)
+    ref = oracle.fftn(np.ascontiguousarray(np.moveaxis(xc, 1, 2)), rank=1, sign=direction, norm=oracle.NORM_ORTHO)
+    assert oracle.rel_l2(np.moveaxis(got.reshape(batch, n, inner), 1, 2), ref) < TOL[dtype]
+
+
+@pytest.mark.parametrize("dtype", ["c32", "c16f"])
+@pytest.mark.parametrize("n,inner", [(n, i) for n in (32, 64, 128, 256, 512, 1024)
+                                     for i in (8, 16, 32, 128, 256, 1 << 14, 1 << 17)])
+def test_rule_matches_the_general_kernels(dtype, n, inner):
+    # strides that fill whole tiles and strides that do not, enough elements
+    # for the rule to choose the tile kernels where it may
+    total = 1 << (25 if dtype == "c32" else 22)
+    batch = max(1, total // (n * inner))
+    general = (16 if n >= 128 and n != 512 else 8, 0)
+    g = torch.Generator(device="cuda").manual_seed(n + inner)
+    x = torch.randn(batch, n, inner, 2, generator=g, device="cuda")
+    x = torch.view_as_complex(x) if dtype == "c32" else x.half()
+    a = _axis(x, dtype, n, inner, batch, W.FORWARD, None)
+    b = _axis(x, dtype, n, inner, batch, W.FORWARD, general)
+    a, b = (torch.view_as_real(t).double() if dtype == "c32" else t.double() for t in (a, b))
+    assert ((a - b).norm() / b.norm()).item() < TOL[dtype]
