@@ -98,6 +98,8 @@ struct Plan {
     const float2 *tc_table(int N);  // tensor-core contiguous superstep (tc_contig.cuh)
     std::map<int64_t, float2 *> fs_tables;        // four-step twiddle tables per long length
     const float2 *fourstep_table(int64_t L, int shift);
+    std::map<std::pair<int64_t, int>, float2 *> fs_tile_tables;  // per long length and first superstep's length
+    const float2 *fourstep_tile_table(int64_t L, int N);
     int build_schedule();
     bool overrides_launchable() const;  // every pass-shape override names an instantiated kernel
     int build_engine(int64_t n0, int64_t n, bool inv);

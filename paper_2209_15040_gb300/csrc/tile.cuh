@@ -72,9 +72,23 @@ struct TileAxis {
 template <int TBITS, int NB>
 struct TileStrided : TileAxis<TBITS, NB> {
     static constexpr int LBUF = (1 << TBITS);
-    static constexpr int ROWBITS = TileAxis<TBITS, NB>::LW, XROWS = 1 << NB;  // elements per row, rows
     __host__ __device__ static constexpr int pair(int) { return 0; }
     __host__ __device__ static constexpr int ls(int slot) { return 1 << slot; }
+};
+
+// Contiguous axis, transposed store: 2^LW whole pencils are copied, and leave
+// as rows of 2^LW elements.  The first stage pairs neighbouring points, the
+// second neighbouring pencils.  EB: bytes of a stored element.
+template <int TBITS, int NB, int EB>
+struct TileTrans : TileAxis<TBITS, NB> {
+    using A = TileAxis<TBITS, NB>;
+    static constexpr int LW = A::LW;
+    // elements between pencils in the load buffer: 16 bytes more than the
+    // pencil, so the first stage's lanes (pencils) spread over the banks
+    static constexpr int PITCH = A::N + 16 / EB;
+    static constexpr int LBUF = PITCH * A::W;
+    __host__ __device__ static constexpr int pair(int s) { return s == 0 ? LW : 0; }
+    __host__ __device__ static constexpr int ls(int slot) { return slot < LW ? PITCH << slot : 1 << (slot - LW); }
 };
 
 // Slot j of the thread index: the slots that are neither in a register nor
@@ -211,6 +225,15 @@ __device__ __forceinline__ void tile_exchange(cpair (&v)[32], float *xw, float *
     tile_part<G, E, E + 1, true, false>(v, xr + IM);
 }
 
+// Product of two split pairs of complex numbers, lane by lane.
+__device__ __forceinline__ cpair cmul(cpair a, cpair w) {
+    return {__ffma2_rn(a.re, w.re, f2neg(__fmul2_rn(a.im, w.im))), __ffma2_rn(a.re, w.im, __fmul2_rn(a.im, w.re))};
+}
+__device__ __forceinline__ cpair ld_cpair(const float4 *p) {
+    const float4 t = *p;
+    return {make_float2(t.x, t.y), make_float2(t.z, t.w)};
+}
+
 // A stage: the digit's twiddles and its DFT.  The twiddles multiply all
 // values before the first butterfly (interleaved with the butterflies the
 // compiler's schedule was 10% slower).
@@ -239,21 +262,25 @@ __device__ __forceinline__ void tile_stage(cpair (&v)[32], const float2 *__restr
 }
 
 // Shared memory: load buffer, exchange buffer (the same bytes in tiles of
-// 2^13 elements), then (16-bit storage) the stage twiddles.
-template <class G, class S>
+// 2^13 elements), then (16-bit storage) the stage twiddles, then (inter-step
+// twiddle) one table per digit of k, for two tiles.
+template <class G, class S, int MODE>
 struct TileSmem {
-    static constexpr int CTAS = G::TB == 14 ? 1 : sizeof(S) == 4 ? 3 : 2;  // blocks per SM
+    static constexpr bool TWID = MODE == TILE_STRIDED_TWID;
+    static constexpr int CTAS = G::TB == 14 ? 1 : sizeof(S) == 4 && !TWID ? 3 : 2;  // blocks per SM
     static constexpr bool SHARED_BUF = G::TB < 14;
     // both parts of an exchange at once where there is room (16-bit tiles of
     // 2^14: 2-4% faster)
-    static constexpr bool FULL = SHARED_BUF || sizeof(S) == 4;
+    static constexpr bool FULL = SHARED_BUF || (sizeof(S) == 4 && !TWID);
     static constexpr int LOAD = G::LBUF * (int)sizeof(S), XCHG = tile_xfloats<G>() * (FULL ? 8 : 4);
     static constexpr int X = SHARED_BUF ? 0 : LOAD;
     static constexpr int TW = SHARED_BUF ? (LOAD > XCHG ? LOAD : XCHG) : LOAD + XCHG;
     // 16-bit storage is bound by the SM and reads its stage twiddles 5%
     // faster from shared memory; complex64 is bound by HBM and was slower so
     static constexpr bool SHARED_TW = sizeof(S) == 4;
-    static constexpr int BYTES = TW + (SHARED_TW ? G::TABLE * 8 : 0);
+    static constexpr int C = TW + (SHARED_TW ? G::TABLE * 8 : 0);
+    static constexpr int TILE_C = TWID ? G::W * (8 << G::R0) : 0, TILE_U = TWID ? G::W * (8 << G::R1) : 0;
+    static constexpr int BYTES = C + 2 * (TILE_C + TILE_U);
     static_assert(BYTES <= 228 * 1024 / CTAS - 1024, "blocks per SM");
 };
 
@@ -267,10 +294,19 @@ struct TileSmem {
 //   16-bit storage: the SM -- FP32 pipe and shared memory, which the blocks
 //     of an SM overlap in part: 512 points 0.20 ms (tiles of 2^13), 0.227
 //     (2^14) against 0.26-0.27; 256 points 0.187 and 0.205 against 0.24-0.25.
-template <class G, class S>
-__global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S>::CTAS)
-    tile_strided_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
-    using SM = TileSmem<G, S>;
+// With the four-step's inter-step twiddle w_L^(q k) on the store (pencil q,
+// k = k1 + Ns r): the product of w_L^(q k1) and w_(L/Ns)^(q r), whose tables
+// hold every q for the few values of k1 and of r, so a tile copies its own
+// columns of both beside its elements and a pair reads them as one 16-byte
+// value (gathered element by element instead: 40% slower).  complex64 1024
+// points 0.344 ms against 0.41-0.53, 16-bit 512 points 0.246 against 0.55.
+// Transposed store of a contiguous axis (the four-step's second superstep and
+// the other spectral layouts): complex64 1024 points 0.389 ms against 0.45-
+// 0.51, 16-bit 512 points 0.214 against 0.305.
+template <class G, class S, int MODE>
+__global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
+    tile_axis_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
+    using SM = TileSmem<G, S, MODE>;
     using PT = typename SplitPair<S>::T;
     constexpr int NT = 1 << (G::TB - 6);
     constexpr bool LDG = !SM::SHARED_TW;
@@ -288,25 +324,49 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S>::CTAS)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int64_t ntiles = a.tiles;
 
-    // first element of a tile
+    // first element of a tile in `in`
     auto tile_base = [&](int64_t t) -> int64_t {
         const int64_t q = (a.reverse ? ntiles - 1 - t : t) * G::W;
-        return ((q >> a.log_inner) * ((int64_t)G::N << a.log_inner)) + (q & (a.inner - 1));
+        if constexpr (MODE == TILE_TRANS) return q * G::N;
+        else return ((q >> a.log_inner) * ((int64_t)G::N << a.log_inner)) + (q & (a.inner - 1));
     };
-    auto issue = [&](int64_t tile) {
-        constexpr int EPC = 16 / (int)sizeof(S), CPR = G::W / EPC, ROWS = NT / CPR;  // chunks per row, rows per round
-        static_assert(CPR <= NT && G::N % ROWS == 0, "whole rounds");
-        const S *p = in + tile_base(tile) + (int64_t)(tid / CPR) * a.inner + (tid % CPR) * EPC;
-        const int64_t step = (int64_t)ROWS * a.inner;
+    constexpr int EPC = 16 / (int)sizeof(S);  // elements per 16-byte chunk
+    auto issue = [&](int64_t tile, int half) {
+        const int64_t base = tile_base(tile);
+        if constexpr (MODE == TILE_TRANS) {
+            constexpr int CPP = G::N / EPC;  // chunks per pencil
 #pragma unroll
-        for (int j = 0; j < G::N / ROWS; ++j) {
-            cp_async16(sm + (tid + j * NT) * 16, p);
-            p += step;
+            for (int c = tid; c < CPP * G::W; c += NT)
+                cp_async16(sm + (c / CPP) * (G::PITCH * (int)sizeof(S)) + (c % CPP) * 16, in + base + (int64_t)c * EPC);
+        } else {
+            constexpr int CPR = G::W / EPC, ROWS = NT / CPR;  // chunks per row, rows per round
+            static_assert(CPR <= NT && G::N % ROWS == 0, "whole rounds");
+            const S *p = in + base + (int64_t)(tid / CPR) * a.inner + (tid % CPR) * EPC;
+            const int64_t step = (int64_t)ROWS * a.inner;
+#pragma unroll
+            for (int j = 0; j < G::N / ROWS; ++j) {
+                cp_async16(sm + (tid + j * NT) * 16, p);
+                p += step;
+            }
+        }
+        if constexpr (MODE == TILE_STRIDED_TWID) {
+            constexpr int CW = G::W / 2, TR = NT / CW, Ns = 1 << G::R0, R = 1 << G::R1;  // pairs per row, rows per round
+            const int qp = ((int)(base & (a.inner - 1)) >> 1) + tid % CW, row = tid / CW;
+            const int half_inner = (int)(a.inner >> 1);
+            const float4 *tc = reinterpret_cast<const float4 *>(a.tw_hi) + qp;
+            const float4 *tu = reinterpret_cast<const float4 *>(a.tw_lo) + qp;
+            char *cu = sm + SM::C + half * (SM::TILE_C + SM::TILE_U) + tid * 16;
+#pragma unroll
+            for (int i = 0; i < Ns; i += TR)
+                if (Ns >= TR || row < Ns) cp_async16(cu + i * CW * 16, tc + (row + i) * half_inner);
+#pragma unroll
+            for (int i = 0; i < R; i += TR)
+                if (R >= TR || row < R) cp_async16(cu + SM::TILE_C + i * CW * 16, tu + (row + i) * half_inner);
         }
     };
     // start the copies of the tile after `tile`
-    auto next = [&](int64_t tile) {
-        if (tile + gridDim.x < ntiles) issue(tile + gridDim.x);
+    auto next = [&](int64_t tile, int half) {
+        if (tile + gridDim.x < ntiles) issue(tile + gridDim.x, half ^ 1);
         else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         cp_async_commit();
     };
@@ -315,8 +375,11 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S>::CTAS)
     const int slots = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid);
     const int wcol = slots & (G::W - 1), k1 = tile_k_of<G, 1>(slots);
 
+    const int64_t ostride = MODE == TILE_TRANS ? a.trans_rows : a.inner;
+
+    int half = 0;
     int64_t tile = blockIdx.x;
-    if (tile < ntiles) issue(tile);
+    if (tile < ntiles) issue(tile, 0);
     cp_async_commit();
     for (; tile < ntiles; tile += gridDim.x) {
         cpair v[32];
@@ -324,35 +387,52 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S>::CTAS)
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
-            v[r] = SplitPair<S>::load(reinterpret_cast<const PT *>(lbuf + tile_reg_off<G, TILE_OFF_LOAD, 0>(r)));
+            const S *p = lbuf + tile_reg_off<G, TILE_OFF_LOAD, 0>(r);
+            static_assert(G::ls(G::pair(0)) == 1, "a pair is two neighbours in the load buffer");
+            v[r] = SplitPair<S>::load(reinterpret_cast<const PT *>(p));
             v[r].im = __fmul2_rn(v[r].im, f2dup(a.conj_in));
         }
         __syncthreads();
-        if constexpr (!SM::SHARED_BUF) next(tile);
+        if constexpr (!SM::SHARED_BUF) next(tile, half);
         tile_stage<G, 0, LDG>(v, tw, 0);
         tile_exchange<G, 0, SM::FULL>(v, xw, xr);
         if constexpr (SM::SHARED_BUF) {
             __syncthreads();
-            next(tile);
+            next(tile, half);
         }
         tile_stage<G, 1, LDG>(v, tw, slots);
         // row k = k1 + Ns k2: k2 in the registers
         constexpr int Ns = 1 << G::R0, R = 1 << G::R1;
-        S *o = out + tile_base(tile) + (int64_t)k1 * a.inner + wcol;
-        const int64_t step = (int64_t)Ns * a.inner;
+        const int64_t base = tile_base(tile);
+        int64_t ob = base;
+        if constexpr (MODE == TILE_TRANS) {
+            // rows per transform are a multiple of W: a tile's rows share one
+            const int64_t q0 = base / G::N, b = q0 / a.trans_rows;
+            ob = b * G::N * a.trans_rows + (q0 - b * a.trans_rows);
+        }
+        S *o = out + ob + (int64_t)k1 * ostride + wcol;
+        const int64_t step = (int64_t)Ns * ostride;
 #pragma unroll
         for (int i = 0; i < 32; i += R) {
             const int sp = tile_reg_off<G, TILE_OFF_SLOT, 1>(i);
-            S *p = o + (int64_t)tile_k_of<G, 1>(sp) * a.inner + (sp & (G::W - 1));
+            const int kc = tile_k_of<G, 1>(sp), wc = sp & (G::W - 1);
+            S *p = o + (int64_t)kc * ostride + wc;
+            const float4 *cu =
+                reinterpret_cast<const float4 *>(sm + SM::C + half * (SM::TILE_C + SM::TILE_U)) + (wcol + wc) / 2;
+            cpair c;
+            if constexpr (MODE == TILE_STRIDED_TWID) c = ld_cpair(cu + (k1 + kc) * (G::W / 2));
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 cpair z = v[i + r];
+                if constexpr (MODE == TILE_STRIDED_TWID)
+                    z = cmul(z, cmul(c, ld_cpair(cu + SM::TILE_C / 16 + r * (G::W / 2))));
                 z.re = __fmul2_rn(z.re, f2dup(a.sx));
                 z.im = __fmul2_rn(z.im, f2dup(a.sy));
                 SplitPair<S>::store(reinterpret_cast<PT *>(p), z);
                 p += step;
             }
         }
+        half ^= 1;
     }
 }
 

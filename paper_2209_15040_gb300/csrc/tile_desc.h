@@ -7,15 +7,22 @@
 
 namespace wsfft {
 
+// Supersteps of the tile kernels.
+enum {
+    TILE_STRIDED = 0,       // strided axis
+    TILE_STRIDED_TWID = 1,  // strided axis, four-step twiddle on the store
+    TILE_TRANS = 2          // contiguous axis, transposed store
+};
+
 // Values per thread of the twiddle table a tile kernel's axis of length N
 // uses: the radix of its first stage.
 inline int tile_table_E(int N) { return N <= 64 ? 8 : N <= 256 ? 16 : 32; }
 
-// Launch one superstep along a strided axis on the pipelined tile kernels.
-// tb: log2 of the elements per tile.  Returns cudaErrorInvalidValue
+// Launch one superstep on the pipelined tile kernels.  tb: log2 of the
+// elements per tile.  Returns cudaErrorInvalidValue
 // for a shape that is not instantiated or does not divide into whole tiles.
-cudaError_t launch_tile_c32(int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
-cudaError_t launch_tile_c16f(int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
-cudaError_t launch_tile_c16bf(int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_c32(int mode, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_c16f(int mode, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_c16bf(int mode, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 
 }  // namespace wsfft

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "launch_util.h"
 #include "tile.cuh"
@@ -14,16 +15,17 @@ namespace {
 
 // Persistent launch: as many blocks as are resident at once, each taking
 // every grid-size-th tile.  Whole tiles of adjacent pencils only.
-template <int TB, int NB>
-cudaError_t launch_tile_strided(const void *in, void *out, PassArgs a, cudaStream_t st) {
+template <int TB, int NB, int MODE>
+cudaError_t launch_tile_axis(const void *in, void *out, PassArgs a, cudaStream_t st) {
     using S = WSFFT_STORE;
-    using G = TileStrided<TB, NB>;
-    using SM = TileSmem<G, S>;
-    auto kern = tile_strided_kernel<G, S>;
+    using G = std::conditional_t<MODE == TILE_TRANS, TileTrans<TB, NB, (int)sizeof(S)>, TileStrided<TB, NB>>;
+    using SM = TileSmem<G, S, MODE>;
+    auto kern = tile_axis_kernel<G, S, MODE>;
     const cudaError_t attr = set_smem_attr(reinterpret_cast<const void *>(kern), SM::BYTES);
     if (attr != cudaSuccess) return attr;
     if (a.npencils <= 0) return cudaSuccess;
-    if (a.npencils % G::W != 0 || a.inner % G::W != 0) return cudaErrorInvalidValue;
+    if (a.npencils % G::W != 0 || (MODE == TILE_TRANS ? a.trans_rows : a.inner) % G::W != 0)
+        return cudaErrorInvalidValue;
     a.tiles = a.npencils / G::W;
     const int sms = device_sms();
     if (sms <= 0) return cudaErrorInvalidDevice;
@@ -34,17 +36,35 @@ cudaError_t launch_tile_strided(const void *in, void *out, PassArgs a, cudaStrea
 
 }  // namespace
 
-cudaError_t WSFFT_TILE_NAME(int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st) {
-    if (N == 1024 && tb == 14) return launch_tile_strided<14, 10>(in, out, a, st);
-    if constexpr (sizeof(WSFFT_STORE) == 4) {
-        if (N == 512 && tb == 14) return launch_tile_strided<14, 9>(in, out, a, st);
-        if (N == 512 && tb == 13) return launch_tile_strided<13, 9>(in, out, a, st);
-        if (N == 256 && tb == 14) return launch_tile_strided<14, 8>(in, out, a, st);
-        if (N == 256 && tb == 13) return launch_tile_strided<13, 8>(in, out, a, st);
-        if (N == 128 && tb == 13) return launch_tile_strided<13, 7>(in, out, a, st);
-        if (N == 64 && tb == 13) return launch_tile_strided<13, 6>(in, out, a, st);
-        if (N == 32 && tb == 13) return launch_tile_strided<13, 5>(in, out, a, st);
+cudaError_t WSFFT_TILE_NAME(int mode, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st) {
+    constexpr bool half = sizeof(WSFFT_STORE) == 4;
+#define WSFFT_TILE(m, n, b, nb) \
+    if (mode == m && N == n && tb == b) return launch_tile_axis<b, nb, m>(in, out, a, st);
+    WSFFT_TILE(TILE_STRIDED, 1024, 14, 10)
+    WSFFT_TILE(TILE_STRIDED_TWID, 512, 13, 9)
+    WSFFT_TILE(TILE_STRIDED_TWID, 256, 13, 8)
+    if constexpr (!half) {
+        WSFFT_TILE(TILE_STRIDED, 1024, 13, 10)
+        WSFFT_TILE(TILE_STRIDED_TWID, 1024, 13, 10)
+        WSFFT_TILE(TILE_TRANS, 1024, 14, 10)
+    } else {
+        WSFFT_TILE(TILE_STRIDED_TWID, 1024, 14, 10)
+        WSFFT_TILE(TILE_TRANS, 1024, 13, 10)
+        WSFFT_TILE(TILE_STRIDED, 512, 14, 9)
+        WSFFT_TILE(TILE_STRIDED, 512, 13, 9)
+        WSFFT_TILE(TILE_STRIDED, 256, 14, 8)
+        WSFFT_TILE(TILE_STRIDED, 256, 13, 8)
+        WSFFT_TILE(TILE_STRIDED, 128, 13, 7)
+        WSFFT_TILE(TILE_STRIDED, 64, 13, 6)
+        WSFFT_TILE(TILE_STRIDED, 32, 13, 5)
+        WSFFT_TILE(TILE_STRIDED_TWID, 128, 13, 7)
+        WSFFT_TILE(TILE_STRIDED_TWID, 64, 13, 6)
+        WSFFT_TILE(TILE_TRANS, 512, 13, 9)
+        WSFFT_TILE(TILE_TRANS, 256, 13, 8)
+        WSFFT_TILE(TILE_TRANS, 128, 13, 7)
+        WSFFT_TILE(TILE_TRANS, 64, 13, 6)
     }
+#undef WSFFT_TILE
     return cudaErrorInvalidValue;
 }
 

@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <complex>
 #include <cstdlib>
 #include <cstdint>
 #include <cstring>
@@ -42,7 +43,9 @@
 
 namespace wsfft {
 
-float2 host_root(int64_t m, int64_t n) {
+namespace {
+// cos and sin of 2*pi*m/n in long double
+std::pair<long double, long double> host_cos_sin(int64_t m, int64_t n) {
     m %= n;
     if (m < 0) m += n;
     const int64_t o = (8 * m) / n;      // octant
@@ -68,7 +71,18 @@ float2 host_root(int64_t m, int64_t n) {
             default: c = cp; s = -sp; break;  // 7
         }
     }
-    return make_float2((float)c, (float)-s);
+    return {c, s};
+}
+}  // namespace
+
+float2 host_root(int64_t m, int64_t n) {
+    const auto cs = host_cos_sin(m, n);
+    return make_float2((float)cs.first, (float)-cs.second);
+}
+
+std::complex<double> host_root_d(int64_t m, int64_t n) {
+    const auto cs = host_cos_sin(m, n);
+    return {(double)cs.first, (double)-cs.second};
 }
 
 int fill_stage_table(float2 *dst, int cap, int N, int E) {
@@ -188,11 +202,12 @@ cudaError_t launch_slab(int dtype, int n, const void *in, void *out, int64_t nsl
     }
 }
 
-cudaError_t launch_tile(int dtype, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st) {
+cudaError_t launch_tile(int dtype, int mode, int N, int tb, const void *in, void *out, const PassArgs &a,
+                        cudaStream_t st) {
     switch (dtype) {
-        case WSFFT_C32: return launch_tile_c32(N, tb, in, out, a, st);
-        case WSFFT_C16F: return launch_tile_c16f(N, tb, in, out, a, st);
-        default: return launch_tile_c16bf(N, tb, in, out, a, st);
+        case WSFFT_C32: return launch_tile_c32(mode, N, tb, in, out, a, st);
+        case WSFFT_C16F: return launch_tile_c16f(mode, N, tb, in, out, a, st);
+        default: return launch_tile_c16bf(mode, N, tb, in, out, a, st);
     }
 }
 
@@ -200,8 +215,9 @@ cudaError_t launch(int dtype, const PassSpec &p, const void *in, void *out, cons
                    cudaStream_t st) {
     if (p.tile >= PIPE_TILE) {
         // the kernels' stage tables are those of one radix per axis length
-        if (p.kind != PASS_STRIDED || p.variant || p.E != tile_table_E(p.N)) return cudaErrorInvalidValue;
-        return launch_tile(dtype, p.N, p.tile - PIPE_TILE, in, out, a, st);
+        if (p.E != tile_table_E(p.N) || (p.kind != PASS_STRIDED && !p.variant)) return cudaErrorInvalidValue;
+        const int mode = p.kind != PASS_STRIDED ? TILE_TRANS : p.variant ? TILE_STRIDED_TWID : TILE_STRIDED;
+        return launch_tile(dtype, mode, p.N, p.tile - PIPE_TILE, in, out, a, st);
     }
     switch (dtype) {
         case WSFFT_C32: return launch_pass_c32(p.kind, p.N, p.E, p.tile, p.variant, in, out, a, st);
@@ -224,9 +240,12 @@ bool override_usable(int E, int tile, int N) {
 // element stride `inner`, over `total` elements, runs on the pipelined tile
 // kernels; 0: the one-tile-per-block kernels are faster, or the pencils do
 // not fill whole tiles.  Measured per superstep, against those kernels:
-//   complex64: 1024 points from 2^25 elements up (2^25 102-107 us against
-//     99-108, 2^27 351-383 against 374-501; 2^23 26.0 against 23.9: too few
-//     tiles of 128 KB per SM); shorter axes are at the copy rate without them.
+//   complex64, 1024 points (shorter axes are at the copy rate without them):
+//     tiles of 2^13 elements up to a stride of 2^16 elements from 2^22
+//     elements up (2^22 12.4 us against 14.4, 2^24 48-50 against 53-57, 2^25
+//     89-92 against 99-108); for large arrays or wider strides their 64-byte
+//     rows cost too much (2^27: 349-372 us, and 540 at a stride of 2^17) and
+//     tiles of 2^14 (128-byte rows) take over (2^27 351-388 us against 373-467).
 //   16-bit storage: from 2^22 elements up (2^27 170-174 us against 224-273
 //     at 32..128 points, 185-206 against 235-251 at 256, 200-212 against
 //     255-271 at 512, 234-237 against 330-338 at 1024; within 0.5 us of each
@@ -237,13 +256,41 @@ bool override_usable(int E, int tile, int N) {
 int pipe_tile_bits(int dtype, int64_t N, int64_t inner, int64_t total) {
     int tb = 0;
     if (dtype == WSFFT_C32) {
-        if (N == 1024 && total >= ((int64_t)1 << 25)) tb = 14;
+        if (N == 1024 && inner <= ((int64_t)1 << 16) && total < ((int64_t)1 << 27))
+            tb = total >= ((int64_t)1 << 22) ? 13 : 0;
+        else if (N == 1024 && total >= ((int64_t)1 << 25))
+            tb = 14;
     } else if (total >= ((int64_t)1 << 22)) {
         if (N == 32 || N == 64 || N == 128) tb = inner <= ((int64_t)1 << 18) ? 13 : 0;
         if (N == 256 || N == 512) tb = inner < ((int64_t)1 << 17) ? 13 : 14;
         if (N == 1024) tb = 14;
     }
     return tb && inner % (((int64_t)1 << tb) / N) == 0 ? tb : 0;
+}
+
+// the same for the four-step's first superstep (twid: inter-step twiddle on a
+// strided store of `rows` pencils per transform) and for a contiguous
+// superstep with the transposed store.  Measured per 2^27 elements, against
+// the general kernels (whose first superstep takes two table reads and a
+// product per element):
+//   twiddle: complex64 256 points 338 us against 358, 512 364-373 against
+//     402, 1024 344 against 410-530; 16-bit 64..256 points 210-225 against
+//     303-330, 512 246 against 552, 1024 282 against 510 (tiles of 2^14: 327 us
+//     with 32-byte rows).
+//   transposed: complex64 1024 points 389 us against 452-505, shorter axes
+//     equal; 16-bit 64..256 points 189-196 against 240-307, 512 214 against
+//     305, 1024 225 against 389.
+// From 2^22 elements (16-bit) or 2^23 (complex64) up; below, both take as long.
+int pipe_tile_bits_variant(int dtype, int64_t N, int64_t rows, int64_t total, bool twid) {
+    int tb = 0;
+    const bool half = dtype != WSFFT_C32;
+    if (twid) {
+        if (N >= (half ? 64 : 256) && N <= 1024) tb = half && N == 1024 ? 14 : 13;
+    } else {
+        if (N == 1024 || (half && N >= 64 && N <= 512)) tb = half ? 13 : 14;
+    }
+    if (total < (int64_t)1 << (half ? 22 : 23)) tb = 0;
+    return tb && rows % (((int64_t)1 << tb) / N) == 0 ? tb : 0;
 }
 
 // two buffers of `bytes` that share some bytes without being the same buffer
@@ -289,6 +336,47 @@ const float2 *Plan::fourstep_table(int64_t L, int shift) {
         return nullptr;
     }
     fs_tables[L] = d;
+    return d;
+}
+
+// The same twiddles for the pipelined tile kernels' first superstep (length
+// N, stage radices Ns and N/Ns, q < n1 = L/N pencils): w_L^(q k1) for
+// k1 < Ns, then w_(L/Ns)^(q r) for r < N/Ns, rows of n1 values, neighbouring
+// pencils as (re0, re1, im0, im1).  The roots are FP64 products of the two
+// tables' long-double roots (a long-double root for each of the 2^16 entries
+// at L = 2^20 would take the host a second), rounded once.
+const float2 *Plan::fourstep_tile_table(int64_t L, int N) {
+    const auto key = std::make_pair(L, N);
+    auto it = fs_tile_tables.find(key);
+    if (it != fs_tile_tables.end()) return it->second;
+    const int64_t n1 = L / N;
+    const int Ns = tile_table_E(N), shift = (ilog2(L) + 1) / 2;
+    const int64_t low = (int64_t)1 << shift;
+    std::vector<std::complex<double>> hi((size_t)(L >> shift)), lo((size_t)low);
+    for (size_t i = 0; i < hi.size(); ++i) hi[i] = host_root_d((int64_t)i << shift, L);
+    for (size_t i = 0; i < lo.size(); ++i) lo[i] = host_root_d((int64_t)i, L);
+    std::vector<float> h;
+    h.reserve((size_t)(2 * n1 * (Ns + N / Ns)));
+    auto rows = [&](int count, int64_t step) {  // w_L^(step q j), j < count
+        for (int j = 0; j < count; ++j)
+            for (int64_t q = 0; q < n1; q += 2) {
+                std::complex<double> w[2];
+                for (int i = 0; i < 2; ++i) {
+                    const int64_t m = (step * (q + i) * j) & (L - 1);
+                    w[i] = hi[(size_t)(m >> shift)] * lo[(size_t)(m & (low - 1))];
+                }
+                for (double v : {w[0].real(), w[1].real(), w[0].imag(), w[1].imag()}) h.push_back((float)v);
+            }
+    };
+    rows(Ns, 1);
+    rows(N / Ns, Ns);
+    float2 *d = nullptr;
+    if (cudaMalloc(&d, h.size() * sizeof(float)) != cudaSuccess) return nullptr;
+    if (upload(d, h.data(), h.size() * sizeof(float)) != WSFFT_SUCCESS) {
+        cudaFree(d);
+        return nullptr;
+    }
+    fs_tile_tables[key] = d;
     return d;
 }
 
@@ -587,6 +675,14 @@ int Plan::build_schedule() {
         }
     };
 
+    // the same for a transposing contiguous superstep of `rows` pencils per transform
+    auto trans_tile = [&](PassSpec &p, int64_t rows) {
+        if (const int tb = pipe_tile_bits_variant(dtype, p.N, rows, elems * batch, false)) {
+            p.E = tile_table_E(p.N);
+            p.tile = PIPE_TILE + tb;
+        }
+    };
+
     // cluster-fused pass A (the default): the two inner axes equal and built
     // for that edge, and the kernel resident on this device
     if (layout == WSFFT_LAYOUT_NATURAL && r == 3 && engine_mode == 4 && d[1] == d[2] && slab_runs((int)d[1]))
@@ -648,6 +744,7 @@ int Plan::build_schedule() {
                 t.E = 32;  // half a warp per pencil, 16 per block (as in the swapped layout)
                 t.tile = 16;
             }
+            trans_tile(t, rows);
             t.variant = true;
             t.inner = 1;
             t.npencils_per_batch = rows;
@@ -744,6 +841,7 @@ int Plan::build_schedule() {
             t.E = 32;
             t.tile = 16;
         }
+        trans_tile(t, n_c);
         t.variant = true;
         t.inner = 1;
         t.npencils_per_batch = A * n_c;
@@ -792,12 +890,12 @@ int Plan::build_schedule() {
     } else if (r == 1 && d[0] > 4096) {
         const int64_t n = d[0];
         const int lg = ilog2(n);
-        // complex64 at n = 2^20 splits 2048 (contiguous) x 512 (strided)
-        // rather than 1024 x 1024: the 512-point strided superstep with the
-        // inter-step twiddle runs at 1.61 ms per 512 x 2^20 execute against
-        // 2.11 ms for the 1024-point one, the 2048-point contiguous superstep
-        // costs 1.97 against 1.81 ms (3.57 vs 3.91 ms per execute)
-        const int lg1 = (lg == 20 && dtype == WSFFT_C32) ? 11 : (lg + 1) / 2;
+        // complex64 at n = 2^20 below 2^23 elements (where the pipelined tile
+        // kernels do not take over) splits 2048 (contiguous) x 512 (strided)
+        // rather than 1024 x 1024: on the general kernels the 512-point
+        // strided superstep with the inter-step twiddle runs at 0.40 ms per
+        // 2^27 elements against 0.53 for the 1024-point one
+        const int lg1 = (lg == 20 && dtype == WSFFT_C32 && elems * batch < ((int64_t)1 << 23)) ? 11 : (lg + 1) / 2;
         const int64_t n1 = (int64_t)1 << lg1;  // contiguous length
         const int64_t n2 = n / n1;             // strided length
         const float sc = axis_scale(n, dir, norm);
@@ -815,6 +913,10 @@ int Plan::build_schedule() {
             // measured fastest at n = 2^20: 32 values per thread, 16 pencils per block
             a.E = 32;
             a.tile = 16;
+        }
+        if (const int tb = pipe_tile_bits_variant(dtype, n2, n1, elems * batch, true)) {
+            a.E = tile_table_E(a.N);
+            a.tile = PIPE_TILE + tb;
         }
         a.variant = true;
         a.inner = n1;
@@ -840,6 +942,7 @@ int Plan::build_schedule() {
             b.E = 32;
             b.tile = 16;
         }
+        trans_tile(b, n2);
         b.variant = true;
         b.inner = 1;
         b.npencils_per_batch = n2;
@@ -905,7 +1008,8 @@ int Plan::build_schedule() {
         if (p.N > 4096 || !is_pow2(p.N)) return WSFFT_ERR_INVALID_SIZE;
         p.tw = p.tile == TC_TILE ? tc_table(p.N) : table(p.N, p.E);
         if (p.twid_len) {
-            p.tw2 = fourstep_table(p.twid_len, p.twid_shift);
+            p.tw2 = p.tile >= PIPE_TILE ? fourstep_tile_table(p.twid_len, p.N)
+                                        : fourstep_table(p.twid_len, p.twid_shift);
             if (!p.tw2) return WSFFT_ERR_ALLOC;
         }
         if (!p.tw) return WSFFT_ERR_ALLOC;
@@ -1045,7 +1149,10 @@ PassArgs Plan::pass_args(const PassSpec &p, int64_t npencils) const {
     a.sy = p.conj_out ? -p.scale : p.scale;
     a.trans_rows = p.trans_rows;
     a.tw_hi = p.twid_len ? p.tw2 : nullptr;
-    a.tw_lo = p.twid_len ? p.tw2 + (p.twid_len >> p.twid_shift) : nullptr;
+    // the low table follows the high one (the tile kernels': the one over k1)
+    a.tw_lo = !p.twid_len ? nullptr
+              : p.tile >= PIPE_TILE ? p.tw2 + (p.twid_len / p.N) * tile_table_E(p.N)
+                                    : p.tw2 + (p.twid_len >> p.twid_shift);
     a.tw_shift = p.twid_len ? p.twid_shift : 0;
     a.tw_mask = p.twid_len ? (int)(p.twid_len - 1) : 0;
     a.status = d_status;
@@ -1303,6 +1410,7 @@ Plan::~Plan() {
     if (d_ctr) cudaFree(d_ctr);
     for (auto &kv : tables) cudaFree(kv.second);
     for (auto &kv : fs_tables) cudaFree(kv.second);
+    for (auto &kv : fs_tile_tables) cudaFree(kv.second);
     if (work) cudaFree(work);
     if (host_buf) cudaFree(host_buf);
     for (auto e : pipe_ev)

@@ -18,7 +18,7 @@ PIPE = 4000
 # (points, values per thread, log2 elements per tile)
 HALF = [(32, 8, 13), (64, 8, 13), (128, 16, 13), (256, 16, 13), (256, 16, 14), (512, 32, 13), (512, 32, 14),
         (1024, 32, 14)]
-SHAPES = [(d, *s) for d in ("c16f", "c16bf") for s in HALF] + [("c32", 1024, 32, 14)]
+SHAPES = [(d, *s) for d in ("c16f", "c16bf") for s in HALF] + [("c32", 1024, 32, 14), ("c32", 1024, 32, 13)]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -49,7 +49,7 @@ def _axis(x, dtype, n, inner, batch, direction, variant):
 def test_strided_tile_shapes(dtype, n, e, tb, tiles):
     w = (1 << tb) // n
     inner = w if tiles == "one" else 2 * w
-    blocks = torch.cuda.get_device_properties(0).multi_processor_count * (1 if tb == 14 else 3)
+    blocks = torch.cuda.get_device_properties(0).multi_processor_count * (1 if tb == 14 else 2 if dtype == "c32" else 3)
     batch = {"one": 1, "few": 5, "rounds": blocks // 2 + 3}[tiles]
     direction = W.INVERSE if tiles == "few" else W.FORWARD
     xs, xc = seeded((batch, n, inner), 11, "uniform", dtype)
@@ -74,3 +74,42 @@ def test_rule_matches_the_general_kernels(dtype, n, inner):
     b = _axis(x, dtype, n, inner, batch, W.FORWARD, general)
     a, b = (torch.view_as_real(t).double() if dtype == "c32" else t.double() for t in (a, b))
     assert ((a - b).norm() / b.norm()).item() < TOL[dtype]
+
+
+def _plan(x, dtype, dims, direction, batch, layout=W.LAYOUT_NATURAL):
+    plan = W.Plan(dims, DT[dtype], direction, batch, W.NORM_ORTHO)
+    try:
+        plan.set_layout(layout)
+        out = torch.empty_like(x)
+        plan.execute(x.data_ptr(), out.data_ptr())
+        same = x.clone()
+        plan.execute(same.data_ptr(), same.data_ptr())
+        torch.cuda.synchronize()
+    finally:
+        plan.close()
+    assert torch.equal(out, same)
+    return out
+
+
+@pytest.mark.parametrize("dtype,lg", [("c32", g) for g in (16, 17, 18, 19, 20, 21)] +
+                         [("c16f", g) for g in range(13, 22)] + [("c16bf", 18)])
+def test_four_step_tiles(dtype, lg):
+    # one transform more than fills the range the rule starts at, so the last
+    # round of tiles is uneven
+    n = 1 << lg
+    batch = ((1 << (23 if dtype == "c32" else 22)) // n) + 1
+    direction = W.INVERSE if lg % 2 else W.FORWARD
+    xs, xc = seeded((batch, n), 13, "uniform", dtype)
+    got = to_host_c128(_plan(to_device(xs, dtype), dtype, (n,), direction, batch), dtype).reshape(batch, n)
+    ref = oracle.fftn(xc, rank=1, sign=direction, norm=oracle.NORM_ORTHO)
+    assert oracle.rel_l2(got, ref) < TOL[dtype]
+
+
+@pytest.mark.parametrize("dtype,dims", [("c32", (1024, 64)), ("c32", (64, 1024))] +
+                         [("c16f", d) for d in ((128, 64), (64, 128), (256, 512), (512, 256), (1024, 64))])
+def test_swapped_layout_tiles(dtype, dims):
+    batch = (1 << (23 if dtype == "c32" else 22)) // (dims[0] * dims[1]) + 1
+    xs, xc = seeded((batch,) + dims, 17, "uniform", dtype)
+    got = to_host_c128(_plan(to_device(xs, dtype), dtype, dims, W.FORWARD, batch, W.LAYOUT_SWAPPED), dtype)
+    ref = oracle.fftn(xc, rank=2, sign=W.FORWARD, norm=oracle.NORM_ORTHO)
+    assert oracle.rel_l2(got.reshape((batch,) + dims[::-1]), np.swapaxes(ref, 1, 2)) < TOL[dtype]
