@@ -286,7 +286,13 @@ int wsfft_plan_set_pass_variant(wsfft_plan plan, int pass, int values_per_thread
 
 /* Choose the schedule of a rank-3 transform n0 x n x n (n in {128, 256, 512,
  * 1024}, any n0; the pipelined engine needs n0 == n):
- *   0 (default): one launch per superstep (three trips through HBM);
+ *   0 (default): one launch per superstep (three trips through HBM); for
+ *      rank-2 and rank-3 transforms with a last axis of 32..256 points whose
+ *      inner two axes hold at most 2^13 elements those two take one launch and
+ *      one trip, and rank-3 transforms of up to 2^22 elements take two trips
+ *      out of place where their axes allow (in place, from host buffers and
+ *      with a chosen pass shape: one launch per superstep; the results agree
+ *      up to rounding);
  *   4 (n in {256, 512}): two trips through HBM -- one thread-block cluster
  *      per n x n slab runs its z superstep, meets at a cluster barrier, and
  *      runs its y superstep on the slab as the z tiles left it in L2; then
@@ -320,8 +326,12 @@ int wsfft_plan_set_wait_test(wsfft_plan plan, int withhold, int64_t timeout_ns);
  * (WSFFT_SUCCESS or WSFFT_ERR_DEVICE_TIMEOUT).  Errors: CUDA. */
 int wsfft_plan_sync_status(wsfft_plan plan, wsfft_stream stream);
 
-/* Number of passes over the array one execute makes, and the minimum number
- * of bytes one execute reads plus writes in HBM for that schedule. */
+/* Number of passes over the array of the plan's schedule (one per superstep,
+ * or the schedule chosen by wsfft_plan_set_engine), and the minimum number of
+ * bytes one execute reads plus writes in HBM for it.  Device executes of
+ * rank-2 and rank-3 transforms whose inner axes fit on a processor's tile make
+ * one pass less (wsfft_plan_set_engine, mode 0); wsfft_plan_launch_times lists
+ * the launches an execute made. */
 int wsfft_plan_passes(wsfft_plan plan, int *passes, int64_t *bytes_per_execute);
 
 /* Per-launch timing (the paper times compute and communication phases

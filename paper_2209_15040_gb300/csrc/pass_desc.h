@@ -47,6 +47,16 @@ struct PassArgs {
     int reverse;        // strided launches: 1 = blocks take the tiles from the last one down
     // pipelined tiles (tile.cuh)
     int64_t tiles;      // tiles of the launch
+    // fused tiles (tile_fused.cuh)
+    const float2 *tw2;  // stage table of the middle axis
+    int64_t elems;      // elements of the launch (slabs: the last tile may be partial)
+    int64_t row;        // elements per row of the last axis
+    int64_t ystep;      // elements between the rows of one frequency k1 of the middle axis
+    int log_y0;         // log2 of the residue classes of the middle axis' rows
+    int log_row;        // log2(row)
+    int log_cols;       // log2 of the columns (k1, z) of a transform
+    int log_transform;  // log2 of the elements per transform
+    int nk1;            // frequencies k1
 };
 
 // tile codes at or above this select the complex64 pencil-pair strided
@@ -76,6 +86,8 @@ enum PassKind {
     PASS_WP_A = 5,       // warp-per-pencil persistent kernel: z and y of every slab
     PASS_WP_B = 6,       // warp-per-pencil strided superstep: x
     PASS_SLAB_A = 7,     // cluster-fused z and y of every n x n slab (slab_cluster.cuh)
+    PASS_TILE_SLAB = 8,  // tile kernel: z and y (or its first digit) of slabs (tile_fused.cuh)
+    PASS_TILE_OUTER = 9, // tile kernel: the rest of y, and x
 };
 
 // Launch one superstep.  variant: contiguous -> transposed store,

@@ -39,6 +39,9 @@ struct PassSpec {
     int64_t units;               // completion counters used (pass A)
     float c_scale, s_scale;      // pass A: scale after the contiguous / strided superstep
     bool reverse;                // strided: tiles taken from the last one down
+    // fused tile passes (PASS_TILE_SLAB, PASS_TILE_OUTER): log2 of the last
+    // axis, of the rows of a tile, of the outer axis and of the residue classes
+    int zb, yb, xb, y0b;
 };
 
 struct Plan {
@@ -50,6 +53,10 @@ struct Plan {
     int64_t axis_inner = 0;  // > 0: a plan of wsfft_plan_create_axis (one axis of length dims[0], stride axis_inner)
     int dtype = 0, dir = -1, norm = 0;
     std::vector<PassSpec> passes;
+    // the same transform with fused tile passes, for device executes (empty:
+    // none); fused_in_place: also when in == out
+    std::vector<PassSpec> fused;
+    bool fused_in_place = false;
     std::map<int, std::pair<int, int>> overrides;  // pass index -> (E, tile)
     std::map<std::pair<int, int>, float2 *> tables;
     int64_t chunk = 1;        // transforms per workspace-sized chunk
@@ -101,6 +108,10 @@ struct Plan {
     std::map<std::pair<int64_t, int>, float2 *> fs_tile_tables;  // per long length and first superstep's length
     const float2 *fourstep_tile_table(int64_t L, int N);
     int build_schedule();
+    int build_fused(const std::vector<int64_t> &d, bool inv);
+    float2 *device_table(const std::vector<float2> &h);
+    const float2 *table2(int N, int R0);  // two stages of radix R0 and N/R0
+    const float2 *class_table(int n, int classes);  // w_n^(y k), y < classes, k < n/classes
     bool overrides_launchable() const;  // every pass-shape override names an instantiated kernel
     int build_engine(int64_t n0, int64_t n, bool inv);
     int build_slab(int64_t n0, int64_t n, bool inv);

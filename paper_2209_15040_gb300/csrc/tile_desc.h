@@ -25,4 +25,19 @@ cudaError_t launch_tile_c32(int mode, int N, int tb, const void *in, void *out, 
 cudaError_t launch_tile_c16f(int mode, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_c16bf(int mode, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 
+// Fused tile kernels (tile_fused.cuh), tiles of 2^13 elements.
+constexpr int FUSED_TILE_BITS = 13;
+
+// The two inner axes of slabs (2^zb points contiguous, 2^yb rows): whole
+// slabs where zb + yb < 13, in place or not; for zb + yb = 13 the 2^yb rows of
+// each residue class of larger slabs (log_y0 of PassArgs; out of place unless
+// it is 0).  cudaErrorInvalidValue for sizes that are not built.
+cudaError_t launch_tile_slab_c32(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_slab_c16f(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_slab_c16bf(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+// The outer axis (2^xb points) and the 2^y0b residue classes.
+cudaError_t launch_tile_outer_c32(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_outer_c16f(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_outer_c16bf(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+
 }  // namespace wsfft

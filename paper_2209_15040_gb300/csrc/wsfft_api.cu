@@ -5,7 +5,9 @@
 // the 3D sequence z, then the other axes):
 //   rank 2/3: superstep along the contiguous axis (in -> out), then one
 //             superstep per remaining axis, last axis first (out -> out,
-//             each kernel reading and writing the same tile).
+//             each kernel reading and writing the same tile).  Where the
+//             inner axes fit (fused_tile_rule) device executes fuse them:
+//             two axes per trip (Plan::fused).
 //   rank 1, n <= 4096: one contiguous superstep.
 //   rank 1, n > 4096: the long axis is split as a 2D problem n = n1*n2
 //             (Section 8 proposes decomposing large 1D transforms as a
@@ -211,8 +213,20 @@ cudaError_t launch_tile(int dtype, int mode, int N, int tb, const void *in, void
     }
 }
 
+cudaError_t launch_fused(int dtype, const PassSpec &p, const void *in, void *out, const PassArgs &a,
+                         cudaStream_t st) {
+    const bool slab = p.kind == PASS_TILE_SLAB;
+    const int b0 = slab ? p.zb : p.xb, b1 = slab ? p.yb : p.y0b;
+    switch (dtype) {
+        case WSFFT_C32: return (slab ? launch_tile_slab_c32 : launch_tile_outer_c32)(b0, b1, in, out, a, st);
+        case WSFFT_C16F: return (slab ? launch_tile_slab_c16f : launch_tile_outer_c16f)(b0, b1, in, out, a, st);
+        default: return (slab ? launch_tile_slab_c16bf : launch_tile_outer_c16bf)(b0, b1, in, out, a, st);
+    }
+}
+
 cudaError_t launch(int dtype, const PassSpec &p, const void *in, void *out, const PassArgs &a,
                    cudaStream_t st) {
+    if (p.kind == PASS_TILE_SLAB || p.kind == PASS_TILE_OUTER) return launch_fused(dtype, p, in, out, a, st);
     if (p.tile >= PIPE_TILE) {
         // the kernels' stage tables are those of one radix per axis length
         if (p.E != tile_table_E(p.N) || (p.kind != PASS_STRIDED && !p.variant)) return cudaErrorInvalidValue;
@@ -291,6 +305,42 @@ int pipe_tile_bits_variant(int dtype, int64_t N, int64_t rows, int64_t total, bo
     }
     if (total < (int64_t)1 << (half ? 22 : 23)) tb = 0;
     return tb && rows % (((int64_t)1 << tb) / N) == 0 ? tb : 0;
+}
+
+// Whether a rank-2 or rank-3 transform (axes d) runs its inner axes fused on
+// the tile kernels (tile_fused.cuh).  A fused trip replaces two (the inner
+// axes of slabs of up to 2^13 elements) or turns three trips into two, and wins
+// at every size measured, from one small transform (a launch less) to 1 GiB
+// (2^27 elements, complex64 / FP16 storage, us):
+//   64 x 64 batches 329 / 262 against 597 / 464, 32^3 623 / 410 against 962 /
+//   771, 64^3 631 / 431 against 896 / 708; split middle axis: 128^3 684 / 458
+//   against 919 / 734 (one cube 15.3 against 18.9), 64 x 256^2 687 / 474
+//   against 907 / 686 (one of 2^22 elements 26.8 against 27.0).
+// Beyond 2^22 elements per transform the outer pass would need tiles of 2^14
+// elements or rows under 128 bytes (16 elements), both slower than a third trip.
+struct FusedShape {
+    bool use = false, outer = false;
+    int zb = 0, yb = 0, y0b = 0;
+};
+FusedShape fused_tile_rule(const std::vector<int64_t> &d) {
+    FusedShape f;
+    const int r = (int)d.size();
+    if (r < 2) return f;
+    const int64_t n1 = d[r - 2], n2 = d[r - 1];
+    if (n2 < 32 || n2 > 256 || n1 < 32) return f;
+    f.zb = ilog2(n2);
+    const int slab = f.zb + ilog2(n1);
+    if (slab <= FUSED_TILE_BITS) {
+        f.yb = ilog2(n1);
+        f.use = true;
+    } else if (r == 3) {
+        f.yb = FUSED_TILE_BITS - f.zb;
+        f.y0b = slab - FUSED_TILE_BITS;
+        const int xb = ilog2(d[0]);
+        // rows of at least 16 elements, within one row of the last axis (one k1)
+        f.use = f.outer = xb >= 5 && f.y0b <= 4 && xb + f.y0b <= 9 && xb + f.y0b + f.zb >= FUSED_TILE_BITS;
+    }
+    return f;
 }
 
 // two buffers of `bytes` that share some bytes without being the same buffer
@@ -393,6 +443,104 @@ const float2 *Plan::table(int N, int E) {
     }
     tables[key] = d;
     return d;
+}
+
+// A device copy of a host table, owned by the caller's map (null on failure).
+float2 *Plan::device_table(const std::vector<float2> &h) {
+    float2 *d = nullptr;
+    if (cudaMalloc(&d, h.size() * sizeof(float2)) != cudaSuccess) return nullptr;
+    if (upload(d, h.data(), h.size() * sizeof(float2)) != WSFFT_SUCCESS) {
+        cudaFree(d);
+        return nullptr;
+    }
+    return d;
+}
+
+// Twiddles of a two-stage pencil, radix R0 then N/R0: w_N^(r k) at
+// (r-1)*R0 + k, r < N/R0, k < R0.
+const float2 *Plan::table2(int N, int R0) {
+    const auto key = std::make_pair(N, 1000 + R0);
+    auto it = tables.find(key);
+    if (it != tables.end()) return it->second;
+    std::vector<float2> h;
+    for (int r = 1; r < N / R0; ++r)
+        for (int k = 0; k < R0; ++k) h.push_back(host_root((int64_t)r * k, N));
+    h.push_back(make_float2(0.f, 0.f));
+    return tables[key] = device_table(h);
+}
+
+// Twiddles between the two parts of a split axis of n points: w_n^(y k) at
+// (y-1)*(n/classes) + k for the residue classes y.
+const float2 *Plan::class_table(int n, int classes) {
+    const auto key = std::make_pair(n, 2000 + classes);
+    auto it = tables.find(key);
+    if (it != tables.end()) return it->second;
+    std::vector<float2> h;
+    for (int y = 1; y < classes; ++y)
+        for (int k = 0; k < n / classes; ++k) h.push_back(host_root((int64_t)y * k, n));
+    h.push_back(make_float2(0.f, 0.f));
+    return tables[key] = device_table(h);
+}
+
+// Fused schedule of the plan (d: its axes longer than one), beside the one
+// launch per superstep in `passes`: see fused_tile_rule.
+int Plan::build_fused(const std::vector<int64_t> &d, bool inv) {
+    const FusedShape f = fused_tile_rule(d);
+    if (!f.use) return WSFFT_SUCCESS;
+    const int r = (int)d.size();
+    const int64_t n1 = d[r - 2], n2 = d[r - 1], n0 = r == 3 ? d[0] : 1;
+    const int64_t rows = (int64_t)1 << f.yb;
+    PassSpec a{};
+    a.kind = PASS_TILE_SLAB;
+    a.N = (int)n2;
+    a.zb = f.zb;
+    a.yb = f.yb;
+    a.y0b = f.y0b;
+    a.inner = n2;
+    a.transform_elems = elems;
+    a.src = SRC_IN;
+    a.dst = DST_OUT;
+    a.conj_in = inv;
+    a.scale = axis_scale(n2 * rows, dir, norm);
+    a.tw = table((int)n2, 16);
+    a.tw2 = table((int)rows, 32);
+    if (!a.tw || !a.tw2) return WSFFT_ERR_ALLOC;
+    fused.push_back(a);
+    if (f.outer) {
+        PassSpec b{};
+        b.kind = PASS_TILE_OUTER;
+        b.N = (int)n0;
+        b.zb = f.zb;
+        b.yb = f.yb;
+        b.xb = ilog2(n0);
+        b.y0b = f.y0b;
+        b.inner = n1 * n2;
+        b.transform_elems = elems;
+        b.src = SRC_OUT;
+        b.dst = DST_OUT;
+        b.scale = axis_scale(n0 << f.y0b, dir, norm);
+        b.reverse = true;  // the slab pass wrote the last transforms last
+        b.tw = table2((int)n0, 32 >> f.y0b);
+        b.tw2 = class_table((int)n1, 1 << f.y0b);
+        if (!b.tw || !b.tw2) return WSFFT_ERR_ALLOC;
+        fused.push_back(b);
+    } else if (r == 3) {
+        PassSpec b = passes.back();  // x as in the one-launch schedule
+        b.scale = axis_scale(n0, dir, norm);
+        b.reverse = true;
+        fused.push_back(b);
+    }
+    fused.back().conj_out = inv;
+    fused_in_place = f.y0b == 0;
+    if (dtype == WSFFT_C32 && norm != WSFFT_NORM_ORTHO) {
+        double total_scale = 1.0;
+        for (auto &p : fused) {
+            total_scale *= p.scale;
+            p.scale = 1.f;
+        }
+        fused.back().scale = (float)total_scale;
+    }
+    return WSFFT_SUCCESS;
 }
 
 // Two-launch schedule of an n^3 cube on the persistent engine.
@@ -609,6 +757,8 @@ int Plan::build_slab(int64_t n0, int64_t n, bool inv) {
 // (Re)build the pass list from shape, direction and normalisation.
 int Plan::build_schedule() {
     passes.clear();
+    fused.clear();
+    fused_in_place = false;
     std::vector<int64_t> d;
     for (int i = 0; i < rank; ++i)
         if (dims[i] > 1) d.push_back(dims[i]);
@@ -1014,6 +1164,10 @@ int Plan::build_schedule() {
         }
         if (!p.tw) return WSFFT_ERR_ALLOC;
     }
+    if (axis_inner == 0 && layout == WSFFT_LAYOUT_NATURAL && engine_mode == 0 && overrides.empty()) {
+        const int rc = build_fused(d, inv);
+        if (rc != WSFFT_SUCCESS) return rc;
+    }
     if (work_elems > work_cap) {
         if (work) cudaFree(work);
         work = nullptr;
@@ -1041,9 +1195,10 @@ bool Plan::overrides_launchable() const {
 
 int Plan::run(const void *in, void *out, cudaStream_t st) {
     const int64_t eb = elem_bytes(dtype);
+    const bool use_fused = !fused.empty() && (in != out || fused_in_place);
     for (int64_t b0 = 0; b0 < batch; b0 += chunk) {
         const int64_t nb = std::min(chunk, batch - b0);
-        for (const auto &p : passes) {
+        for (const auto &p : use_fused ? fused : passes) {
             if (p.kind == PASS_WP_B) {
                 WpStridedArgs b{};
                 b.in = out;
@@ -1128,7 +1283,8 @@ int Plan::run(const void *in, void *out, cudaStream_t st) {
                               : p.src == SRC_OUT ? (const char *)out + off
                                                  : (const char *)work;
             char *dst = p.dst == DST_OUT ? (char *)out + off : (char *)work;
-            const PassArgs a = pass_args(p, p.npencils_per_batch * nb);
+            PassArgs a = pass_args(p, p.npencils_per_batch * nb);
+            a.elems = p.transform_elems * nb;
             prof_begin(st);
             cudaError_t e = launch(dtype, p, src, dst, a, st);
             prof_end(st);
@@ -1158,6 +1314,18 @@ PassArgs Plan::pass_args(const PassSpec &p, int64_t npencils) const {
     a.status = d_status;
     a.timeout_ns = (uint64_t)wait_timeout_ns;
     a.reverse = p.reverse ? 1 : 0;
+    if (p.kind == PASS_TILE_SLAB) {
+        a.tw2 = p.tw2;
+        a.row = (int64_t)1 << p.zb;
+        a.log_y0 = p.y0b;
+    } else if (p.kind == PASS_TILE_OUTER) {
+        a.tw_hi = p.tw2;
+        a.ystep = (int64_t)1 << (p.zb + p.yb);
+        a.log_row = p.zb;
+        a.log_cols = p.zb + p.yb;
+        a.log_transform = ilog2(p.transform_elems);
+        a.nk1 = 1 << p.yb;
+    }
     return a;
 }
 
