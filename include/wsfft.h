@@ -290,9 +290,10 @@ int wsfft_plan_set_pass_variant(wsfft_plan plan, int pass, int values_per_thread
  *      rank-2 and rank-3 transforms with a last axis of 32..256 points whose
  *      inner two axes hold at most 2^13 elements those two take one launch and
  *      one trip, and rank-3 transforms of up to 2^22 elements take two trips
- *      out of place where their axes allow (in place, from host buffers and
- *      with a chosen pass shape: one launch per superstep; the results agree
- *      up to rounding);
+ *      out of place where their axes allow; a strided axis of 2048 or 4096
+ *      points (or 1024 far apart) gives its first digit to the last axis'
+ *      launch, out of place (in place, from host buffers and with a chosen
+ *      pass shape: one launch per superstep; the results agree up to rounding);
  *   4 (n in {256, 512}): two trips through HBM -- one thread-block cluster
  *      per n x n slab runs its z superstep, meets at a cluster barrier, and
  *      runs its y superstep on the slab as the z tiles left it in L2; then

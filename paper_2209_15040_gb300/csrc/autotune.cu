@@ -162,6 +162,7 @@ std::vector<std::pair<int, int>> shapes_for(int kind, int N, int dtype) {
     if (kind == PASS_CONTIG && N == 512 && dtype != WSFFT_C32)
         return {{32, 16}, {32, 8}, {32, 32}, {16, 8}, {8, 8}, {16, TC_TILE}, {16, SPLIT_TILE + 8},
                 {16, SPLIT_TILE + 16}, {8, SPLIT_TILE + 8}};
+    if (kind == PASS_STRIDED && N >= 2048) return {{16, 0}, {16, PIPE_TILE + 14}};
     if (kind == PASS_STRIDED && N == 512)
         return {{32, 16}, {32, 8},  {32, 32}, {16, 16}, {8, 8}, {16, 8}, {16, 32}, {8, PAIR_TILE + 16},
                 {8, PAIR_TILE + 32}, {8, PAIR_TILE + 8}, {16, PAIR_TILE + 16}, {16, PAIR_TILE + 32},

@@ -88,6 +88,7 @@ enum PassKind {
     PASS_SLAB_A = 7,     // cluster-fused z and y of every n x n slab (slab_cluster.cuh)
     PASS_TILE_SLAB = 8,  // tile kernel: z and y (or its first digit) of slabs (tile_fused.cuh)
     PASS_TILE_OUTER = 9, // tile kernel: the rest of y, and x
+    PASS_TILE_WIDE = 10, // tile kernel: z and one digit of a strided axis
 };
 
 // Launch one superstep.  variant: contiguous -> transposed store,

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <functional>
 #include <map>
 #include <utility>
 #include <vector>
@@ -39,8 +40,8 @@ struct PassSpec {
     int64_t units;               // completion counters used (pass A)
     float c_scale, s_scale;      // pass A: scale after the contiguous / strided superstep
     bool reverse;                // strided: tiles taken from the last one down
-    // fused tile passes (PASS_TILE_SLAB, PASS_TILE_OUTER): log2 of the last
-    // axis, of the rows of a tile, of the outer axis and of the residue classes
+    // fused tile passes (PASS_TILE_*): log2 of the last axis, of the rows of a
+    // tile, of the outer axis and of the residue classes of the rows
     int zb, yb, xb, y0b;
 };
 
@@ -109,6 +110,10 @@ struct Plan {
     const float2 *fourstep_tile_table(int64_t L, int N);
     int build_schedule();
     int build_fused(const std::vector<int64_t> &d, bool inv);
+    using StridedBuilder = std::function<PassSpec(int64_t n, int64_t inner)>;
+    int build_wide(const std::vector<int64_t> &d, bool inv, const StridedBuilder &strided);
+    void defer_scale(std::vector<PassSpec> &list) const;
+    const float2 *wide_table(int zb, int rb);
     float2 *device_table(const std::vector<float2> &h);
     const float2 *table2(int N, int R0);  // two stages of radix R0 and N/R0
     const float2 *class_table(int n, int classes);  // w_n^(y k), y < classes, k < n/classes

@@ -25,6 +25,8 @@
 // pass through a 70 KB exchange buffer one after the other.
 #pragma once
 
+#include <type_traits>
+
 #include "pass_kernels.cuh"
 #include "tile_desc.h"
 
@@ -43,8 +45,9 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 //   pair(s)            slot of the pair
 //   in(s, j)           slot of register bit j (the digit first, then spares)
 //   gbits(s)           bits of the digit
-//   nsbits(s), kslot(s, i)  bits of the frequency so far (0: no twiddle) and
-//                      the slot of its bit i
+//   nsbits(s), kslot(s, i), twoff(s)  bits of the frequency so far (0: no
+//                      twiddle), the slot of its bit i, and where the stage's
+//                      twiddles start in the table
 //   ls(slot), LBUF     load-buffer stride of a slot, elements of the buffer
 
 // Slots of a tile of 2^NB points x 2^(TB-NB) pencils: pencil bits first, then
@@ -59,6 +62,9 @@ struct TileAxis {
     __host__ __device__ static constexpr int gbits(int s) { return s == 0 ? R0 : R1; }
     __host__ __device__ static constexpr int nsbits(int s) { return s == 0 ? 0 : R0; }
     __host__ __device__ static constexpr int kslot(int, int i) { return TBITS - R0 + i; }
+    __host__ __device__ static constexpr int twoff(int) { return 0; }
+    __host__ __device__ static constexpr int nlead(int) { return 0; }
+    __host__ __device__ static constexpr int lead(int, int) { return -1; }
     __host__ __device__ static constexpr int in(int s, int j) {
         if (j < gbits(s)) return (s == 0 ? TBITS - R0 : LW) + j;
         // spares: the top pencil bits (a pencil's exchange then stays in fewer
@@ -68,9 +74,33 @@ struct TileAxis {
     static constexpr int TABLE = ((1 << R1) - 1) << R0;  // entries of the twiddle table
 };
 
+// The same for 2048 and 4096 points: three stages of four, four and the
+// remaining bits.
+template <int TBITS, int NB>
+struct TileLongAxis {
+    static_assert(NB == 11 || NB == 12, "three register stages");
+    static constexpr int LW = TBITS - NB, W = 1 << LW, N = 1 << NB;
+    static constexpr int R0 = 4, R1 = 4, R2 = NB - 8;
+    static constexpr int TB = TBITS;
+    static constexpr int NST = 3;
+    __host__ __device__ static constexpr int gbits(int s) { return s == 2 ? R2 : 4; }
+    __host__ __device__ static constexpr int nsbits(int s) { return 4 * s; }
+    // k = k1 + 16 k2: k1 in the axis' top slots, k2 below them
+    __host__ __device__ static constexpr int kslot(int, int i) { return i < 4 ? TBITS - 4 + i : TBITS - 12 + i; }
+    __host__ __device__ static constexpr int twoff(int s) { return s == 2 ? 15 * 16 : 0; }
+    __host__ __device__ static constexpr int nlead(int) { return 0; }
+    __host__ __device__ static constexpr int lead(int, int) { return -1; }
+    __host__ __device__ static constexpr int in(int s, int j) {
+        if (j < gbits(s)) return (s == 0 ? TBITS - 4 : s == 1 ? TBITS - 8 : LW) + j;
+        // spares: the slot below the first digit, then the top frequency bits
+        return s == 0 ? TBITS - 5 : TBITS - 1 - (j - gbits(s));
+    }
+    static constexpr int TABLE = 15 * 16 + ((1 << R2) - 1) * 256;
+};
+
 // Strided axis: 2^LW adjacent pencils, rows of the tile copied whole.
 template <int TBITS, int NB>
-struct TileStrided : TileAxis<TBITS, NB> {
+struct TileStrided : std::conditional_t<(NB > 10), TileLongAxis<TBITS, (NB > 10 ? NB : 11)>, TileAxis<TBITS, (NB > 10 ? 10 : NB)>> {
     static constexpr int LBUF = (1 << TBITS);
     __host__ __device__ static constexpr int pair(int) { return 0; }
     __host__ __device__ static constexpr int ls(int slot) { return 1 << slot; }
@@ -92,13 +122,16 @@ struct TileTrans : TileAxis<TBITS, NB> {
 };
 
 // Slot j of the thread index: the slots that are neither in a register nor
-// the pair, lowest first.
+// the pair, lowest first -- after those the geometry puts in front (lead),
+// where the lowest frequency bits of the last stage are not the lowest slots.
 template <class G>
 __host__ __device__ constexpr int tile_th(int s, int j) {
-    int c = 0;
+    int c = G::nlead(s);
+    if (j < c) return G::lead(s, j);
     for (int slot = 0; slot < G::TB; ++slot) {
         bool used = slot == G::pair(s);
         for (int i = 0; i < 5; ++i) used |= G::in(s, i) == slot;
+        for (int i = 0; i < G::nlead(s); ++i) used |= G::lead(s, i) == slot;
         if (used) continue;
         if (c == j) return slot;
         ++c;
@@ -241,7 +274,7 @@ template <class G, int SG, bool LDG>
 __device__ __forceinline__ void tile_stage(cpair (&v)[32], const float2 *__restrict__ tw, int slots) {
     constexpr int B = G::gbits(SG), R = 1 << B, NSB = G::nsbits(SG);
     if constexpr (NSB > 0) {
-        const float2 *tk = tw + tile_k_of<G, SG>(slots);
+        const float2 *tk = tw + G::twoff(SG) + tile_k_of<G, SG>(slots);
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
             const int r = i & (R - 1);
@@ -370,10 +403,16 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         cp_async_commit();
     };
+    constexpr int LAST = G::NST - 1;
     const S *lbuf = reinterpret_cast<const S *>(sm) + tile_thread_off<G, TILE_OFF_LOAD, 0>(tid);
     float *xw = xb + tile_thread_off<G, 0, 0>(tid), *xr = xb + tile_thread_off<G, 0, 1>(tid);
-    const int slots = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid);
-    const int wcol = slots & (G::W - 1), k1 = tile_k_of<G, 1>(slots);
+    float *xw1 = xb, *xr1 = xb;
+    if constexpr (LAST == 2) {
+        xw1 += tile_thread_off<G, 1, 1>(tid);
+        xr1 += tile_thread_off<G, 1, 2>(tid);
+    }
+    const int slots1 = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid), slots = tile_thread_off<G, TILE_OFF_SLOT, LAST>(tid);
+    const int wcol = slots & (G::W - 1), k1 = tile_k_of<G, LAST>(slots);
 
     const int64_t ostride = MODE == TILE_TRANS ? a.trans_rows : a.inner;
 
@@ -396,13 +435,17 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         if constexpr (!SM::SHARED_BUF) next(tile, half);
         tile_stage<G, 0, LDG>(v, tw, 0);
         tile_exchange<G, 0, SM::FULL>(v, xw, xr);
+        if constexpr (LAST == 2) {
+            tile_stage<G, 1, LDG>(v, tw, slots1);
+            tile_exchange<G, 1, SM::FULL>(v, xw1, xr1);
+        }
         if constexpr (SM::SHARED_BUF) {
             __syncthreads();
             next(tile, half);
         }
-        tile_stage<G, 1, LDG>(v, tw, slots);
-        // row k = k1 + Ns k2: k2 in the registers
-        constexpr int Ns = 1 << G::R0, R = 1 << G::R1;
+        tile_stage<G, LAST, LDG>(v, tw, slots);
+        // row k = k1 + Ns r: the last digit r in the registers
+        constexpr int Ns = 1 << G::nsbits(LAST), R = 1 << G::gbits(LAST);
         const int64_t base = tile_base(tile);
         int64_t ob = base;
         if constexpr (MODE == TILE_TRANS) {
@@ -414,8 +457,8 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         const int64_t step = (int64_t)Ns * ostride;
 #pragma unroll
         for (int i = 0; i < 32; i += R) {
-            const int sp = tile_reg_off<G, TILE_OFF_SLOT, 1>(i);
-            const int kc = tile_k_of<G, 1>(sp), wc = sp & (G::W - 1);
+            const int sp = tile_reg_off<G, TILE_OFF_SLOT, LAST>(i);
+            const int kc = tile_k_of<G, LAST>(sp), wc = sp & (G::W - 1);
             S *p = o + (int64_t)kc * ostride + wc;
             const float4 *cu =
                 reinterpret_cast<const float4 *>(sm + SM::C + half * (SM::TILE_C + SM::TILE_U)) + (wcol + wc) / 2;

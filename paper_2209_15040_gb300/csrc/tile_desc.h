@@ -16,7 +16,7 @@ enum {
 
 // Values per thread of the twiddle table a tile kernel's axis of length N
 // uses: the radix of its first stage.
-inline int tile_table_E(int N) { return N <= 64 ? 8 : N <= 256 ? 16 : 32; }
+inline int tile_table_E(int N) { return N <= 64 ? 8 : N <= 256 || N >= 2048 ? 16 : 32; }
 
 // Launch one superstep on the pipelined tile kernels.  tb: log2 of the
 // elements per tile.  Returns cudaErrorInvalidValue
@@ -35,6 +35,11 @@ constexpr int FUSED_TILE_BITS = 13;
 cudaError_t launch_tile_slab_c32(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_slab_c16f(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_slab_c16bf(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+// A last axis of 2^zb = 512..4096 points and a digit of 2^rb points of a
+// strided axis; out of place.
+cudaError_t launch_tile_wide_c32(int zb, int rb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_wide_c16f(int zb, int rb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_wide_c16bf(int zb, int rb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 // The outer axis (2^xb points) and the 2^y0b residue classes.
 cudaError_t launch_tile_outer_c32(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_outer_c16f(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);

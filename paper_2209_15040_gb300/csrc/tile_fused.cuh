@@ -25,8 +25,8 @@ namespace wsfft {
 // ---------------------------------------------------------------------------
 // Geometries with several digits per stage:
 //   ngroups(s), gbits(s, g)   digits of a stage and their bits
-//   nsbits(s, g), kslot(s, g, i), tbl(s, g)   frequency so far on the digit's
-//                             axis, its slots, and the twiddle table
+//   nsbits(s, g), kslot(s, g, i)   frequency so far on the digit's axis, its slots
+//   tbl(s, g), twoff(s, g)    the twiddle table and where the stage's start in it
 
 // 2^YB rows of 2^ZB contiguous elements, transformed along both; spare slots
 // above are further such slabs.  Three stages: the high five bits of y; the
@@ -54,6 +54,9 @@ struct TileSlab {
     __host__ __device__ static constexpr int nsbits(int s, int g) { return s < 2 ? 0 : g == 0 ? 4 : 5; }
     __host__ __device__ static constexpr int kslot(int, int g, int i) { return (g == 0 ? C2 : ZB + YL) + i; }
     __host__ __device__ static constexpr int tbl(int, int g) { return g; }
+    __host__ __device__ static constexpr int twoff(int, int) { return 0; }
+    __host__ __device__ static constexpr int nlead(int) { return 0; }
+    __host__ __device__ static constexpr int lead(int, int) { return -1; }
     static constexpr int TABLE0 = ((1 << C2) - 1) << 4, TABLE1 = ((1 << YL) - 1) << 5;
 };
 
@@ -78,7 +81,41 @@ struct TileOuter {
     __host__ __device__ static constexpr int nsbits(int s, int) { return s == 0 ? 0 : XH; }
     __host__ __device__ static constexpr int kslot(int, int, int i) { return LW + XL + i; }
     __host__ __device__ static constexpr int tbl(int, int) { return 0; }
+    __host__ __device__ static constexpr int twoff(int, int) { return 0; }
+    __host__ __device__ static constexpr int nlead(int) { return 0; }
+    __host__ __device__ static constexpr int lead(int, int) { return -1; }
     static constexpr int TABLE0 = ((1 << XL) - 1) << XH, TABLE1 = 0;
+};
+
+// 2^(TB-ZB) rows of 2^ZB contiguous elements (512..4096), transformed along
+// the row and, in one digit, across the rows.  Three stages: the high ZA bits
+// of z and the rows; the next five bits of z; the low ZC bits.
+template <int TBITS, int ZB>
+struct TileWide {
+    static constexpr int RB = TBITS - ZB, ZA = 5 - RB, ZC = TBITS - 10;
+    static_assert(RB >= 1 && RB <= 4 && ZA + 5 + ZC == ZB, "three register stages");
+    static constexpr int TB = TBITS;
+    static constexpr int NST = 3;
+    static constexpr int LBUF = (1 << TBITS);
+    __host__ __device__ static constexpr int pair(int s) { return s == 2 ? ZB - ZA : 0; }
+    __host__ __device__ static constexpr int ls(int slot) { return 1 << slot; }
+    __host__ __device__ static constexpr int ngroups(int s) { return s == 0 ? 2 : 1; }
+    __host__ __device__ static constexpr int gbits(int s, int g) { return s == 0 ? (g == 0 ? ZA : RB) : s == 1 ? 5 : ZC; }
+    __host__ __device__ static constexpr int in(int s, int j) {
+        if (s == 0) return TBITS - 5 + j;
+        if (s == 1) return ZC + j;
+        if (j < ZC) return j;
+        return j - ZC < RB ? TBITS - 1 - (j - ZC) : ZC + 4 - (j - ZC - RB);  // spares: rows, then z's second digit
+    }
+    __host__ __device__ static constexpr int nsbits(int s, int) { return s == 0 ? 0 : s == 1 ? ZA : ZA + 5; }
+    // kz = k1 + 2^ZA k2 (+ 2^(ZA+5) k3)
+    __host__ __device__ static constexpr int kslot(int, int, int i) { return i < ZA ? ZB - ZA + i : ZC + i - ZA; }
+    __host__ __device__ static constexpr int tbl(int, int) { return 0; }
+    __host__ __device__ static constexpr int twoff(int s, int) { return s == 2 ? 31 << ZA : 0; }
+    // the store's lanes: the rest of k1, then k2
+    __host__ __device__ static constexpr int nlead(int s) { return s == 2 ? ZA - 1 : 0; }
+    __host__ __device__ static constexpr int lead(int, int i) { return ZB - ZA + 1 + i; }
+    static constexpr int TABLE0 = (31 << ZA) + (((1 << ZC) - 1) << (ZA + 5)), TABLE1 = 0;
 };
 
 // frequency so far on a group's axis that a set of slots holds
@@ -103,7 +140,7 @@ template <class G, int SG, int GR, bool LDG>
 __device__ __forceinline__ void tile_group(cpair (&v)[32], const float2 *__restrict__ tw, int slots) {
     constexpr int LO = tile_group_lo<G>(SG, GR), B = G::gbits(SG, GR), R = 1 << B, NSB = G::nsbits(SG, GR);
     if constexpr (NSB > 0) {
-        const float2 *tk = tw + tile_gk_of<G, SG, GR>(slots);
+        const float2 *tk = tw + G::twoff(SG, GR) + tile_gk_of<G, SG, GR>(slots);
         // the pair may be the lowest bit of k: two neighbouring twiddles
         constexpr bool two = G::kslot(SG, GR, 0) == G::pair(SG);
 #pragma unroll
@@ -136,14 +173,17 @@ __device__ __forceinline__ void tile_gstage(cpair (&v)[32], const float2 *tw0, c
     if constexpr (G::ngroups(SG) > 1) tile_group<G, SG, 1, LDG>(v, G::tbl(SG, 1) ? tw1 : tw0, slots);
 }
 
-// Shared memory: the load buffer, which the exchanges run through, then
-// (16-bit storage) the stage twiddles.
+// Shared memory: load buffer, exchange buffer (the same bytes in tiles of
+// 2^13 elements), then (16-bit storage, tables of up to 8 KB) the stage
+// twiddles.
 template <class G, class S>
 struct TileFusedSmem {
-    static constexpr int CTAS = sizeof(S) == 4 ? 3 : 2;  // blocks per SM
-    static constexpr int LOAD = G::LBUF * (int)sizeof(S), XCHG = tile_xfloats<G>() * 8;
-    static constexpr bool SHARED_TW = sizeof(S) == 4;
-    static constexpr int TW = LOAD > XCHG ? LOAD : XCHG;
+    static constexpr int CTAS = G::TB == 14 ? 1 : sizeof(S) == 4 ? 3 : 2;  // blocks per SM
+    static constexpr bool SHARED_BUF = G::TB < 14, FULL = SHARED_BUF || sizeof(S) == 4;
+    static constexpr int LOAD = G::LBUF * (int)sizeof(S), XCHG = tile_xfloats<G>() * (FULL ? 8 : 4);
+    static constexpr bool SHARED_TW = sizeof(S) == 4 && G::TABLE0 + G::TABLE1 <= 1024;
+    static constexpr int X = SHARED_BUF ? 0 : LOAD;
+    static constexpr int TW = SHARED_BUF ? (LOAD > XCHG ? LOAD : XCHG) : LOAD + XCHG;
     static constexpr int BYTES = TW + (SHARED_TW ? (G::TABLE0 + G::TABLE1) * 8 : 0);
     static_assert(BYTES <= 228 * 1024 / CTAS - 1024, "blocks per SM");
 };
@@ -358,6 +398,98 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
                 tile_store(p, v[i + r], a);
                 p += step;
             }
+        }
+    }
+}
+
+// One digit of a strided axis of n points (element stride a.inner, a multiple
+// of the row) beside the last axis: tile (o, y0, j) takes rows y1 Y0 + y0
+// (Y0 = n/2^RB, j: which row of the axis' stride), and frequency k1 leaves,
+// times w_n^(y0 k1), at R y0 + k1.  What is left of the axis is a strided
+// superstep of Y0 points at R times the stride.  Bound by the SM (three stages
+// over 13 bits: complex64 0.36-0.37 ms per 2^27 elements, 0.85 of the copy
+// rate; 16-bit storage 0.285-0.295); with 4096-point rows and a radix of 4,
+// tiles of 2^14 elements: 0.485 and 0.37.
+template <class G, class S>
+__global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
+    tile_wide_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
+    using SM = TileFusedSmem<G, S>;
+    constexpr int NT = 1 << (G::TB - 6), ZB = G::TB - G::RB;
+    constexpr bool LDG = !SM::SHARED_TW;
+    extern __shared__ float4 t_smem[];
+    char *sm = reinterpret_cast<char *>(t_smem);
+    float *xb = reinterpret_cast<float *>(sm + SM::X);
+    const int tid = threadIdx.x;
+    const float2 *tw0, *tw1;
+    tile_tables<G, S>(sm, a, tw0, tw1);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int64_t ntiles = a.tiles;
+
+    const int log_m = a.log_inner - ZB;  // rows within the axis' stride
+    auto y0_of = [&](int64_t tile) { return (tile >> log_m) & (((int64_t)1 << a.log_y0) - 1); };
+    // first element of (o, y0 << shift, j)
+    auto tile_base = [&](int64_t tile, int shift) -> int64_t {
+        const int64_t o = tile >> (log_m + a.log_y0), j = tile & (((int64_t)1 << log_m) - 1);
+        return (((o << (a.log_y0 + G::RB)) + (y0_of(tile) << shift)) << a.log_inner) + (j << ZB);
+    };
+    auto issue = [&](int64_t tile) {
+        constexpr int EPC = 16 / (int)sizeof(S), PER = (1 << ZB) / EPC / NT;  // rounds per row
+        static_assert(PER >= 1, "a row takes whole rounds");
+        const S *src = in + tile_base(tile, 0) + tid * EPC;
+        const int64_t rs = a.inner << a.log_y0;
+#pragma unroll
+        for (int y = 0; y < (1 << G::RB); ++y) {
+#pragma unroll
+            for (int j = 0; j < PER; ++j) cp_async16(sm + (tid + (y * PER + j) * NT) * 16, src + j * NT * EPC);
+            src += rs;
+        }
+    };
+    auto next = [&](int64_t tile) {
+        if (tile + gridDim.x < ntiles) issue(tile + gridDim.x);
+        else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        cp_async_commit();
+    };
+    const S *lbuf = reinterpret_cast<const S *>(sm) + tile_thread_off<G, TILE_OFF_LOAD, 0>(tid);
+    float *xw0 = xb + tile_thread_off<G, 0, 0>(tid), *xr0 = xb + tile_thread_off<G, 0, 1>(tid);
+    float *xw1 = xb + tile_thread_off<G, 1, 1>(tid), *xr1 = xb + tile_thread_off<G, 1, 2>(tid);
+    const int slots1 = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid), slots2 = tile_thread_off<G, TILE_OFF_SLOT, 2>(tid);
+    // frequency along the row; the digit's sits in the slots above
+    auto kz = [](int s) constexpr -> int {
+        const int k1 = (s >> (ZB - G::ZA)) & ((1 << G::ZA) - 1), k2 = (s >> G::ZC) & 31, k3 = s & ((1 << G::ZC) - 1);
+        return k1 + (k2 << G::ZA) + (k3 << (G::ZA + 5));
+    };
+    const int64_t to = (int64_t)(slots2 >> ZB) * a.inner + kz(slots2);
+
+    int64_t tile = blockIdx.x;
+    if (tile < ntiles) issue(tile);
+    cp_async_commit();
+    for (; tile < ntiles; tile += gridDim.x) {
+        cpair v[32];
+        cp_async_wait_all();
+        __syncthreads();
+        tile_load<G, S>(v, lbuf, a.conj_in);
+        __syncthreads();
+        if constexpr (!SM::SHARED_BUF) next(tile);
+        tile_gstage<G, 0, LDG>(v, tw0, tw1, 0);
+        const float2 *wy = a.tw_hi + y0_of(tile);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const int k = i >> G::ZA;
+            if (k > 0) v[i] = cmul(v[i], __ldg(wy + ((int64_t)(k - 1) << a.log_y0)));
+        }
+        tile_exchange<G, 0, SM::FULL>(v, xw0, xr0);
+        tile_gstage<G, 1, LDG>(v, tw0, tw1, slots1);
+        tile_exchange<G, 1, SM::FULL>(v, xw1, xr1);
+        if constexpr (SM::SHARED_BUF) {
+            __syncthreads();
+            next(tile);
+        }
+        tile_gstage<G, 2, LDG>(v, tw0, tw1, slots2);
+        S *o = out + tile_base(tile, G::RB) + to;
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+            const int sp = tile_reg_off<G, TILE_OFF_SLOT, 2>(r);
+            tile_store(o + (int64_t)(sp >> ZB) * a.inner + kz(sp), v[r], a);
         }
     }
 }

@@ -52,6 +52,23 @@ cudaError_t WSFFT_SLAB_TILE_NAME(int zb, int yb, const void *in, void *out, cons
 }
 #endif
 
+#ifdef WSFFT_WIDE_TILE_NAME
+cudaError_t WSFFT_WIDE_TILE_NAME(int zb, int rb, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
+    using S = WSFFT_STORE;
+    PassArgs a = arg;
+    a.tiles = a.elems >> (zb + rb);
+#define WSFFT_WIDE(b, z) \
+    if (zb == z && rb == b - z) return launch_fused<TileWide<b, z>>(tile_wide_kernel<TileWide<b, z>, S>, in, out, a, st);
+    WSFFT_WIDE(13, 9)
+    WSFFT_WIDE(13, 10)
+    WSFFT_WIDE(13, 11)
+    WSFFT_WIDE(13, 12)
+    WSFFT_WIDE(14, 12)
+#undef WSFFT_WIDE
+    return cudaErrorInvalidValue;
+}
+#endif
+
 #ifdef WSFFT_OUTER_TILE_NAME
 cudaError_t WSFFT_OUTER_TILE_NAME(int xb, int y0b, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
     using S = WSFFT_STORE;

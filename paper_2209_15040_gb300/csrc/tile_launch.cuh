@@ -41,6 +41,7 @@ cudaError_t WSFFT_TILE_NAME(int mode, int N, int tb, const void *in, void *out, 
 #define WSFFT_TILE(m, n, b, nb) \
     if (mode == m && N == n && tb == b) return launch_tile_axis<b, nb, m>(in, out, a, st);
     WSFFT_TILE(TILE_STRIDED, 1024, 14, 10)
+    WSFFT_TILE(TILE_STRIDED, 2048, 14, 11)
     WSFFT_TILE(TILE_STRIDED_TWID, 512, 13, 9)
     WSFFT_TILE(TILE_STRIDED_TWID, 256, 13, 8)
     if constexpr (!half) {
@@ -50,6 +51,7 @@ cudaError_t WSFFT_TILE_NAME(int mode, int N, int tb, const void *in, void *out, 
     } else {
         WSFFT_TILE(TILE_STRIDED_TWID, 1024, 14, 10)
         WSFFT_TILE(TILE_TRANS, 1024, 13, 10)
+        WSFFT_TILE(TILE_STRIDED, 4096, 14, 12)
         WSFFT_TILE(TILE_STRIDED, 512, 14, 9)
         WSFFT_TILE(TILE_STRIDED, 512, 13, 9)
         WSFFT_TILE(TILE_STRIDED, 256, 14, 8)

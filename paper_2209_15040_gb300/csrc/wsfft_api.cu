@@ -215,18 +215,18 @@ cudaError_t launch_tile(int dtype, int mode, int N, int tb, const void *in, void
 
 cudaError_t launch_fused(int dtype, const PassSpec &p, const void *in, void *out, const PassArgs &a,
                          cudaStream_t st) {
-    const bool slab = p.kind == PASS_TILE_SLAB;
-    const int b0 = slab ? p.zb : p.xb, b1 = slab ? p.yb : p.y0b;
-    switch (dtype) {
-        case WSFFT_C32: return (slab ? launch_tile_slab_c32 : launch_tile_outer_c32)(b0, b1, in, out, a, st);
-        case WSFFT_C16F: return (slab ? launch_tile_slab_c16f : launch_tile_outer_c16f)(b0, b1, in, out, a, st);
-        default: return (slab ? launch_tile_slab_c16bf : launch_tile_outer_c16bf)(b0, b1, in, out, a, st);
-    }
+    using Fn = cudaError_t (*)(int, int, const void *, void *, const PassArgs &, cudaStream_t);
+    static constexpr Fn slab[3] = {launch_tile_slab_c32, launch_tile_slab_c16f, launch_tile_slab_c16bf};
+    static constexpr Fn outer[3] = {launch_tile_outer_c32, launch_tile_outer_c16f, launch_tile_outer_c16bf};
+    static constexpr Fn wide[3] = {launch_tile_wide_c32, launch_tile_wide_c16f, launch_tile_wide_c16bf};
+    if (p.kind == PASS_TILE_OUTER) return outer[dtype](p.xb, p.y0b, in, out, a, st);
+    return (p.kind == PASS_TILE_SLAB ? slab : wide)[dtype](p.zb, p.yb, in, out, a, st);
 }
 
 cudaError_t launch(int dtype, const PassSpec &p, const void *in, void *out, const PassArgs &a,
                    cudaStream_t st) {
-    if (p.kind == PASS_TILE_SLAB || p.kind == PASS_TILE_OUTER) return launch_fused(dtype, p, in, out, a, st);
+    if (p.kind == PASS_TILE_SLAB || p.kind == PASS_TILE_OUTER || p.kind == PASS_TILE_WIDE)
+        return launch_fused(dtype, p, in, out, a, st);
     if (p.tile >= PIPE_TILE) {
         // the kernels' stage tables are those of one radix per axis length
         if (p.E != tile_table_E(p.N) || (p.kind != PASS_STRIDED && !p.variant)) return cudaErrorInvalidValue;
@@ -254,6 +254,9 @@ bool override_usable(int E, int tile, int N) {
 // element stride `inner`, over `total` elements, runs on the pipelined tile
 // kernels; 0: the one-tile-per-block kernels are faster, or the pencils do
 // not fill whole tiles.  Measured per superstep, against those kernels:
+//   2048 points, three stages, 64-byte rows (complex64): 508-587 us against
+//     566-603, 16-bit 383-431 against 466-481; 4096 points only in 16-bit storage
+//     (583-662 against 631-704; complex64 732 against 696).
 //   complex64, 1024 points (shorter axes are at the copy rate without them):
 //     tiles of 2^13 elements up to a stride of 2^16 elements from 2^22
 //     elements up (2^22 12.4 us against 14.4, 2^24 48-50 against 53-57, 2^25
@@ -269,6 +272,8 @@ bool override_usable(int E, int tile, int N) {
 //     2^16 elements and 282 at 2^18, where tiles of 2^14 take 210 and 212.
 int pipe_tile_bits(int dtype, int64_t N, int64_t inner, int64_t total) {
     int tb = 0;
+    if (N == 2048) tb = total >= ((int64_t)1 << 22) ? 14 : 0;
+    if (N == 4096 && dtype != WSFFT_C32) tb = total >= ((int64_t)1 << 23) ? 14 : 0;
     if (dtype == WSFFT_C32) {
         if (N == 1024 && inner <= ((int64_t)1 << 16) && total < ((int64_t)1 << 27))
             tb = total >= ((int64_t)1 << 22) ? 13 : 0;
@@ -341,6 +346,40 @@ FusedShape fused_tile_rule(const std::vector<int64_t> &d) {
         f.use = f.outer = xb >= 5 && f.y0b <= 4 && xb + f.y0b <= 9 && xb + f.y0b + f.zb >= FUSED_TILE_BITS;
     }
     return f;
+}
+
+// Whether a rank-2 or rank-3 transform out of place runs a digit of a long
+// strided axis in the trip of its last axis (tile_wide_kernel): axis (-1: none)
+// and the digit's bits.  Strided supersteps of 2048 and 4096 points have
+// rows of 32-64 bytes and one block per SM (0.55 and 0.45 of the copy rate in
+// complex64, 0.35 and 0.26 in 16-bit storage), those of 1024 points rows that lie
+// megabytes apart; what is left of the axis after the digit is a superstep at
+// the copy rate, for a last-axis trip of 0.36-0.37 ms per 2^27 elements
+// (complex64) instead of 0.30-0.35.  Measured (complex64 / FP16, us): 4096^2
+// 123 / 85 against 141 / 117 (8 of them 843 / 609 against 1064 / 899), 32 x
+// 2048^2 684 / 495 against 889 / 741, 64 x 2048 x 1024 677 / 470 against 870 /
+// 827, 1024^3 8100 / 5982 against 8766 / 7126, 1024 x 512^2 1997 against 2107;
+// 1024 x 128 x 1024, whose outer stride is 2^17, 996 / 701 against 986 / 649.
+// Below 2^20 elements (2^21 in 16-bit storage) the three-stage tile's latency
+// costs more (one FP16 2048 x 512: 14.3 against 13.2).
+struct WideShape {
+    int axis = -1, rb = 0;
+};
+WideShape wide_tile_rule(int dtype, const std::vector<int64_t> &d, int64_t total) {
+    WideShape w;
+    const int r = (int)d.size();
+    if (r < 2 || total < ((int64_t)1 << (dtype == WSFFT_C32 ? 20 : 21))) return w;
+    const int zb = ilog2(d[r - 1]);
+    if (zb < 9 || zb > 12) return w;
+    // the longest of the axes that qualify; the outer one where both are as long
+    for (int ax = r - 2; ax >= 0; --ax) {
+        const bool far = r == 3 && ax == 0 && d[0] == 1024 && d[1] * d[2] >= ((int64_t)1 << 18);
+        if ((d[ax] >= 2048 || far) && (w.axis < 0 || d[ax] >= d[w.axis])) w.axis = ax;
+    }
+    if (w.axis < 0) return w;
+    // tiles of 2^13 elements; of 2^14 only where a radix of 2 would leave 2048 points
+    w.rb = zb == 12 && d[w.axis] == 4096 ? 2 : 13 - zb;
+    return w;
 }
 
 // two buffers of `bytes` that share some bytes without being the same buffer
@@ -482,6 +521,74 @@ const float2 *Plan::class_table(int n, int classes) {
     return tables[key] = device_table(h);
 }
 
+// Stage twiddles of the 2^zb points of a wide tile (TileWide): radices
+// 2^(5-rb), 32 and the rest.
+const float2 *Plan::wide_table(int zb, int rb) {
+    const auto key = std::make_pair(1 << zb, 3000 + rb);
+    auto it = tables.find(key);
+    if (it != tables.end()) return it->second;
+    std::vector<float2> h;
+    int64_t ns = (int64_t)1 << (5 - rb);
+    for (int R : {32, (1 << zb) / (32 << (5 - rb))}) {
+        for (int r = 1; r < R; ++r)
+            for (int64_t k = 0; k < ns; ++k) h.push_back(host_root(r * k, ns * R));
+        ns *= R;
+    }
+    return tables[key] = device_table(h);
+}
+
+// Schedule with one digit of a long strided axis in the trip of the last
+// axis: see wide_tile_rule.  `strided` builds the superstep of an axis of n
+// points at element stride `inner`.
+int Plan::build_wide(const std::vector<int64_t> &d, bool inv, const StridedBuilder &strided) {
+    const int r = (int)d.size();
+    const WideShape w = wide_tile_rule(dtype, d, elems * batch);
+    if (w.axis < 0) return WSFFT_SUCCESS;
+    std::vector<int64_t> inner((size_t)r, 1);
+    for (int ax = r - 2; ax >= 0; --ax) inner[ax] = inner[ax + 1] * d[ax + 1];
+    const int64_t n = d[w.axis], R = (int64_t)1 << w.rb;
+    PassSpec a{};
+    a.kind = PASS_TILE_WIDE;
+    a.N = (int)d[r - 1];
+    a.zb = ilog2(d[r - 1]);
+    a.yb = w.rb;
+    a.y0b = ilog2(n / R);
+    a.inner = inner[w.axis];
+    a.transform_elems = elems;
+    a.src = SRC_IN;
+    a.dst = DST_OUT;
+    a.conj_in = inv;
+    a.scale = axis_scale(d[r - 1] * R, dir, norm);
+    a.tw = wide_table(a.zb, a.yb);
+    a.tw2 = class_table((int)n, (int)R);
+    if (!a.tw || !a.tw2) return WSFFT_ERR_ALLOC;
+    fused.push_back(a);
+    for (int ax = r - 2; ax >= 0; --ax) {
+        const bool split = ax == w.axis;
+        PassSpec p = strided(split ? n / R : d[ax], split ? R * inner[ax] : inner[ax]);
+        p.reverse = ax == r - 2;
+        p.tw = table(p.N, p.E);
+        if (!p.tw) return WSFFT_ERR_ALLOC;
+        fused.push_back(p);
+    }
+    fused.back().conj_out = inv;
+    defer_scale(fused);
+    return WSFFT_SUCCESS;
+}
+
+// complex64 has the range to defer every superstep's scale to the last store
+// (one scaled store instead of one per pass); the reduced-precision types and
+// the orthonormal scaling keep the per-superstep scale.
+void Plan::defer_scale(std::vector<PassSpec> &list) const {
+    if (dtype != WSFFT_C32 || norm == WSFFT_NORM_ORTHO) return;
+    double total_scale = 1.0;
+    for (auto &p : list) {
+        total_scale *= p.scale;
+        p.scale = 1.f;
+    }
+    list.back().scale = (float)total_scale;
+}
+
 // Fused schedule of the plan (d: its axes longer than one), beside the one
 // launch per superstep in `passes`: see fused_tile_rule.
 int Plan::build_fused(const std::vector<int64_t> &d, bool inv) {
@@ -532,14 +639,7 @@ int Plan::build_fused(const std::vector<int64_t> &d, bool inv) {
     }
     fused.back().conj_out = inv;
     fused_in_place = f.y0b == 0;
-    if (dtype == WSFFT_C32 && norm != WSFFT_NORM_ORTHO) {
-        double total_scale = 1.0;
-        for (auto &p : fused) {
-            total_scale *= p.scale;
-            p.scale = 1.f;
-        }
-        fused.back().scale = (float)total_scale;
-    }
+    defer_scale(fused);
     return WSFFT_SUCCESS;
 }
 
@@ -1165,7 +1265,22 @@ int Plan::build_schedule() {
         if (!p.tw) return WSFFT_ERR_ALLOC;
     }
     if (axis_inner == 0 && layout == WSFFT_LAYOUT_NATURAL && engine_mode == 0 && overrides.empty()) {
-        const int rc = build_fused(d, inv);
+        int rc = build_fused(d, inv);
+        if (rc == WSFFT_SUCCESS && fused.empty())
+            rc = build_wide(d, inv, [&](int64_t n, int64_t inner) {
+                PassSpec p{};
+                p.kind = PASS_STRIDED;
+                p.N = (int)n;
+                p.E = default_E(p.N);
+                tune(p, inner);
+                p.inner = inner;
+                p.npencils_per_batch = elems / n;
+                p.src = SRC_OUT;
+                p.dst = DST_OUT;
+                p.scale = axis_scale(n, dir, norm);
+                p.transform_elems = elems;
+                return p;
+            });
         if (rc != WSFFT_SUCCESS) return rc;
     }
     if (work_elems > work_cap) {
@@ -1317,6 +1432,9 @@ PassArgs Plan::pass_args(const PassSpec &p, int64_t npencils) const {
     if (p.kind == PASS_TILE_SLAB) {
         a.tw2 = p.tw2;
         a.row = (int64_t)1 << p.zb;
+        a.log_y0 = p.y0b;
+    } else if (p.kind == PASS_TILE_WIDE) {
+        a.tw_hi = p.tw2;
         a.log_y0 = p.y0b;
     } else if (p.kind == PASS_TILE_OUTER) {
         a.tw_hi = p.tw2;

@@ -94,3 +94,43 @@ def test_normalisations_match_the_unfused_schedule(norm):
             torch.cuda.synchronize()
             plan.close()
             assert ((fused - plain).norm() / plain.norm()).item() < TOL["c32"]
+
+
+# a long strided axis beside a last axis of 512..4096 points: each row length,
+# the digit taken from the middle axis, from the outer one, and (4096 x 4096) a
+# tile of 2^14 elements
+WIDE = [((2048, 512), 2), ((4096, 1024), 2), ((2048, 2048), 2), ((2048, 4096), 2), ((4096, 4096), 2),
+        ((2, 4096, 512), 3), ((2048, 2, 1024), 3), ((4096, 4, 512), 3), ((1024, 512, 512), 3)]
+
+
+@pytest.mark.parametrize("dtype", ["c32", "c16f", "c16bf"])
+@pytest.mark.parametrize("dims,passes", WIDE)
+def test_digit_of_a_long_axis(dtype, dims, passes):
+    n = 1
+    for v in dims:
+        n *= v
+    if n > 1 << 24 and dtype == "c16bf":
+        pytest.skip("the largest shape in two storage types")
+    batch = max(1, (1 << 21) // n)
+    _check(dims, batch, dtype, W.FORWARD if len(dims) == 2 else W.INVERSE, passes)
+
+
+def test_axes_outside_the_wide_rule():
+    # the general kernels and the wide tiles agree on the shapes next to the
+    # rule's limits, whichever of them runs
+    for dtype, dims, batch in [("c32", (2048, 256), 2), ("c32", (2048, 512), 1), ("c16f", (2048, 512), 1),
+                               ("c16f", (2048, 512), 2), ("c32", (1024, 256, 512), 1), ("c32", (1024, 4096), 1)]:
+        xs, xc = seeded((batch,) + dims, 31, "uniform", dtype)
+        x = to_device(xs, dtype)
+        outs = []
+        for chosen in (False, True):
+            plan = W.Plan(dims, DT[dtype], W.FORWARD, batch, W.NORM_ORTHO)
+            if chosen:  # any chosen shape: one launch per superstep
+                e = 8 if dims[-1] == 512 else 16
+                plan.set_pass_variant(0, e, 8 if e == 8 else 0)
+            out = torch.empty_like(x)
+            plan.execute(x.data_ptr(), out.data_ptr())
+            torch.cuda.synchronize()
+            plan.close()
+            outs.append(to_host_c128(out, dtype))
+        assert oracle.rel_l2(outs[0], outs[1]) < TOL[dtype]

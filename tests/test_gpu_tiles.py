@@ -17,8 +17,9 @@ pytestmark = pytest.mark.gpu
 PIPE = 4000
 # (points, values per thread, log2 elements per tile)
 HALF = [(32, 8, 13), (64, 8, 13), (128, 16, 13), (256, 16, 13), (256, 16, 14), (512, 32, 13), (512, 32, 14),
-        (1024, 32, 14)]
-SHAPES = [(d, *s) for d in ("c16f", "c16bf") for s in HALF] + [("c32", 1024, 32, 14), ("c32", 1024, 32, 13)]
+        (1024, 32, 14), (2048, 16, 14), (4096, 16, 14)]
+SHAPES = [(d, *s) for d in ("c16f", "c16bf") for s in HALF] + [("c32", 1024, 32, 14), ("c32", 1024, 32, 13),
+                                                                      ("c32", 2048, 16, 14)]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -59,7 +60,7 @@ def test_strided_tile_shapes(dtype, n, e, tb, tiles):
 
 
 @pytest.mark.parametrize("dtype", ["c32", "c16f"])
-@pytest.mark.parametrize("n,inner", [(n, i) for n in (32, 64, 128, 256, 512, 1024)
+@pytest.mark.parametrize("n,inner", [(n, i) for n in (32, 64, 128, 256, 512, 1024, 2048, 4096)
                                      for i in (8, 16, 32, 128, 256, 1 << 14, 1 << 17)])
 def test_rule_matches_the_general_kernels(dtype, n, inner):
     # strides that fill whole tiles and strides that do not, enough elements
