@@ -173,6 +173,8 @@ std::vector<std::pair<int, int>> shapes_for(int kind, int N, int dtype) {
     if (kind == PASS_CONTIG && N == 512)
         return {{32, 16}, {32, 8}, {32, 32}, {16, 8}, {8, 8}, {16, SPLIT_TILE + 8}, {16, SPLIT_TILE + 16}};
     if (kind == PASS_CONTIG && N == 256) return {{8, 8}};
+    if (kind == PASS_CONTIG && (N == 32 || N == 64)) return {{8, 0}, {8, PIPE_TILE + 13}};
+    if (kind == PASS_CONTIG && N == 128) return {{16, 0}, {16, PIPE_TILE + 13}};
     return {};
 }
 

@@ -35,6 +35,10 @@ constexpr int FUSED_TILE_BITS = 13;
 cudaError_t launch_tile_slab_c32(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_slab_c16f(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_slab_c16bf(int zb, int yb, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+// Contiguous pencils of N = 32, 64 or 128 points, any number of them, in place or not.
+cudaError_t launch_tile_contig_c32(int N, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_contig_c16f(int N, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_tile_contig_c16bf(int N, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 // A last axis of 2^zb = 512..4096 points and a digit of 2^rb points of a
 // strided axis; out of place.
 cudaError_t launch_tile_wide_c32(int zb, int rb, const void *in, void *out, const PassArgs &a, cudaStream_t st);

@@ -42,6 +42,7 @@ struct TileSlab {
     static constexpr int LBUF = (1 << TBITS);
     __host__ __device__ static constexpr int pair(int s) { return s == 2 ? C2 : 0; }
     __host__ __device__ static constexpr int ls(int slot) { return 1 << slot; }
+    __host__ __device__ static constexpr int chunk_at(int c, int) { return c * 16; }
     __host__ __device__ static constexpr int ngroups(int s) { return s == 2 && YL > 0 ? 2 : 1; }
     __host__ __device__ static constexpr int gbits(int s, int g) { return s == 0 ? 5 : s == 1 ? 4 : g == 0 ? C2 : YL; }
     __host__ __device__ static constexpr int in(int s, int j) {
@@ -58,6 +59,51 @@ struct TileSlab {
     __host__ __device__ static constexpr int nlead(int) { return 0; }
     __host__ __device__ static constexpr int lead(int, int) { return -1; }
     static constexpr int TABLE0 = ((1 << C2) - 1) << 4, TABLE1 = ((1 << YL) - 1) << 5;
+    // where a slot's frequencies leave: z = kz1 + 16 kz2, y = ky1 + 32 ky2
+    __host__ __device__ static constexpr int place(int s) {
+        const int kz = ((s >> C2) & 15) | ((s & ((1 << C2) - 1)) << 4);
+        const int y = s >> ZB;
+        const int ky = ((y >> YL) & 31) | ((y & ((1 << YL) - 1)) << 5);
+        return kz + (ky << ZB) + ((y >> YB) << (ZB + YB));
+    }
+};
+
+// Contiguous axis of 2^NB points, whole pencils: the high R0 bits, then the
+// low R1 bits.  The last stage's pair is the lowest frequency bit and its lanes
+// run over the rest of the first digit: whole runs of a pencil per access.
+template <int TBITS, int NB>
+struct TileContig {
+    static_assert(NB >= 5 && NB <= 8, "two register stages");
+    static constexpr int R0 = NB >= 7 ? 4 : 3, R1 = NB - R0;
+    static constexpr int TB = TBITS;
+    static constexpr int NST = 2;
+    // elements between pencils in the load buffer: the first stage's lanes
+    // (2^R1 neighbours, then pencils) spread over the banks
+    static constexpr int PITCH = (1 << NB) + (1 << R1);
+    static constexpr int LBUF = PITCH << (TBITS - NB);
+    __host__ __device__ static constexpr int pair(int s) { return s == 0 ? 0 : R1; }
+    __host__ __device__ static constexpr int ls(int slot) { return slot < NB ? 1 << slot : PITCH << (slot - NB); }
+    // byte in the load buffer of the tile's 16-byte chunk c
+    __host__ __device__ static constexpr int chunk_at(int c, int eb) {
+        const int per = (1 << NB) * eb / 16;
+        return (c / per) * (PITCH * eb) + (c % per) * 16;
+    }
+    __host__ __device__ static constexpr int ngroups(int) { return 1; }
+    __host__ __device__ static constexpr int gbits(int s, int) { return s == 0 ? R0 : R1; }
+    __host__ __device__ static constexpr int in(int s, int j) {
+        const int b = s == 0 ? R0 : R1;
+        return j < b ? (s == 0 ? R1 : 0) + j : TBITS - 1 - (j - b);  // spares: the top pencil bits
+    }
+    __host__ __device__ static constexpr int nsbits(int s, int) { return s == 0 ? 0 : R0; }
+    __host__ __device__ static constexpr int kslot(int, int, int i) { return R1 + i; }
+    __host__ __device__ static constexpr int tbl(int, int) { return 0; }
+    __host__ __device__ static constexpr int twoff(int, int) { return 0; }
+    __host__ __device__ static constexpr int nlead(int) { return 0; }
+    __host__ __device__ static constexpr int lead(int, int) { return -1; }
+    static constexpr int TABLE0 = ((1 << R1) - 1) << R0, TABLE1 = 0;
+    __host__ __device__ static constexpr int place(int s) {
+        return ((s >> R1) & ((1 << R0) - 1)) + ((s & ((1 << R1) - 1)) << R0) + ((s >> NB) << NB);
+    }
 };
 
 // The outer axis (2^XB points) and the low Y0B bits of the middle one, whose
@@ -227,7 +273,9 @@ __device__ __forceinline__ void tile_store(S *p, cpair z, const PassArgs &a) {
 // blocks per SM (three in 16-bit storage) of 2^13 elements rather than one of
 // 2^14: three stages in one block leave FP32 pipe and shared memory idle in
 // turn (0.43-0.48 ms).
-// WHOLE: tiles of whole slabs of 2^(ZB+YB) < 2^13 elements (the last tile may
+// Contiguous pencils alone (TileContig): 16-bit storage 32 / 64 / 128 points
+// 0.197 / 0.192 / 0.194 ms against 0.341 / 0.234 / 0.263.
+// WHOLE: tiles of whole slabs (or pencils) of 2^(ZB+YB) < 2^13 elements (the last tile may
 // be partial); otherwise the rows of one residue class of a slab of 2^13
 // << a.log_y0 elements.
 template <class G, class S, bool WHOLE>
@@ -237,6 +285,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     constexpr int NT = 1 << (G::TB - 6), ELEMS = 1 << G::TB;
     constexpr int EPC = 16 / (int)sizeof(S), CHUNKS = ELEMS / EPC;  // elements per 16-byte chunk, chunks per tile
     constexpr bool LDG = !SM::SHARED_TW;
+    constexpr int LAST = G::NST - 1;
     extern __shared__ float4 t_smem[];
     char *sm = reinterpret_cast<char *>(t_smem);
     float *xb = reinterpret_cast<float *>(sm);
@@ -252,11 +301,13 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
             const S *src = in + base + tid * EPC;
             if (left >= ELEMS) {
 #pragma unroll
-                for (int j = 0; j < CHUNKS / NT; ++j) cp_async16(sm + (tid + j * NT) * 16, src + j * NT * EPC);
+                for (int j = 0; j < CHUNKS / NT; ++j)
+                    cp_async16(sm + G::chunk_at(tid + j * NT, (int)sizeof(S)), src + j * NT * EPC);
             } else {
 #pragma unroll 1
                 for (int j = 0; j < CHUNKS / NT; ++j)
-                    if ((tid + j * NT) * EPC < left) cp_async16(sm + (tid + j * NT) * 16, src + j * NT * EPC);
+                    if ((tid + j * NT) * EPC < left)
+                        cp_async16(sm + G::chunk_at(tid + j * NT, (int)sizeof(S)), src + j * NT * EPC);
             }
         } else {
             // slab tile >> log_y0, rows y0, y0 + Y0, ...
@@ -275,16 +326,13 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     };
     const S *lbuf = reinterpret_cast<const S *>(sm) + tile_thread_off<G, TILE_OFF_LOAD, 0>(tid);
     float *xw0 = xb + tile_thread_off<G, 0, 0>(tid), *xr0 = xb + tile_thread_off<G, 0, 1>(tid);
-    float *xw1 = xb + tile_thread_off<G, 1, 1>(tid), *xr1 = xb + tile_thread_off<G, 1, 2>(tid);
-    const int slots1 = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid), slots2 = tile_thread_off<G, TILE_OFF_SLOT, 2>(tid);
-    // place of a slot's frequencies in the slab: z = kz1 + 16 kz2, y = ky1 + 32 ky2
-    auto place = [](int s) constexpr -> int {
-        const int kz = ((s >> G::C2) & 15) | ((s & ((1 << G::C2) - 1)) << 4);
-        const int y = s >> (G::C2 + 4);
-        const int ky = ((y >> G::YL) & 31) | ((y & ((1 << G::YL) - 1)) << 5);
-        return kz + (ky << (G::C2 + 4)) + ((y >> (G::YL + 5)) << (G::C2 + 4 + G::YL + 5));
-    };
-    const int to = place(slots2);
+    float *xw1 = xb, *xr1 = xb;
+    if constexpr (LAST == 2) {
+        xw1 += tile_thread_off<G, 1, 1>(tid);
+        xr1 += tile_thread_off<G, 1, 2>(tid);
+    }
+    const int slots1 = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid), slots2 = tile_thread_off<G, TILE_OFF_SLOT, LAST>(tid);
+    const int to = G::place(slots2);
 
     int64_t tile = blockIdx.x;
     if (tile < ntiles) issue(tile);
@@ -297,13 +345,15 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         __syncthreads();
         tile_gstage<G, 0, LDG>(v, tw0, tw1, 0);
         tile_exchange<G, 0, true>(v, xw0, xr0);
-        tile_gstage<G, 1, LDG>(v, tw0, tw1, slots1);
-        tile_exchange<G, 1, true>(v, xw1, xr1);
+        if constexpr (LAST == 2) {
+            tile_gstage<G, 1, LDG>(v, tw0, tw1, slots1);
+            tile_exchange<G, 1, true>(v, xw1, xr1);
+        }
         __syncthreads();
         if (tile + gridDim.x < ntiles) issue(tile + gridDim.x);
         else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         cp_async_commit();
-        tile_gstage<G, 2, LDG>(v, tw0, tw1, slots2);
+        tile_gstage<G, LAST, LDG>(v, tw0, tw1, slots2);
         const int64_t base = tile << G::TB;
         S *o = out + base + to;
         int lim = ELEMS;
@@ -311,7 +361,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
             if (a.elems - base < ELEMS) lim = (int)(a.elems - base) - to;
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
-            const int at = place(tile_reg_off<G, TILE_OFF_SLOT, 2>(r));
+            const int at = G::place(tile_reg_off<G, TILE_OFF_SLOT, LAST>(r));
             if (!WHOLE || at < lim) tile_store(o + at, v[r], a);
         }
     }

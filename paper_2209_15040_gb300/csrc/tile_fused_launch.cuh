@@ -52,6 +52,24 @@ cudaError_t WSFFT_SLAB_TILE_NAME(int zb, int yb, const void *in, void *out, cons
 }
 #endif
 
+#ifdef WSFFT_CONTIG_TILE_NAME
+cudaError_t WSFFT_CONTIG_TILE_NAME(int N, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
+    using S = WSFFT_STORE;
+    PassArgs a = arg;
+    a.elems = a.npencils * N;
+    a.tiles = (a.elems + (1 << FUSED_TILE_BITS) - 1) >> FUSED_TILE_BITS;
+#define WSFFT_CONTIG(n, b)                                                                                          \
+    if (N == n)                                                                                                     \
+        return launch_fused<TileContig<FUSED_TILE_BITS, b>>(tile_slab_kernel<TileContig<FUSED_TILE_BITS, b>, S, true>, in, \
+                                                            out, a, st);
+    WSFFT_CONTIG(32, 5)
+    WSFFT_CONTIG(64, 6)
+    WSFFT_CONTIG(128, 7)
+#undef WSFFT_CONTIG
+    return cudaErrorInvalidValue;
+}
+#endif
+
 #ifdef WSFFT_WIDE_TILE_NAME
 cudaError_t WSFFT_WIDE_TILE_NAME(int zb, int rb, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
     using S = WSFFT_STORE;

@@ -114,3 +114,28 @@ def test_swapped_layout_tiles(dtype, dims):
     got = to_host_c128(_plan(to_device(xs, dtype), dtype, dims, W.FORWARD, batch, W.LAYOUT_SWAPPED), dtype)
     ref = oracle.fftn(xc, rank=2, sign=W.FORWARD, norm=oracle.NORM_ORTHO)
     assert oracle.rel_l2(got.reshape((batch,) + dims[::-1]), np.swapaxes(ref, 1, 2)) < TOL[dtype]
+
+
+@pytest.mark.parametrize("dtype", ["c32", "c16f", "c16bf"])
+@pytest.mark.parametrize("n,e", [(32, 8), (64, 8), (128, 16)])
+def test_contiguous_tiles(dtype, n, e):
+    # one pencil, a partial tile, whole tiles, a partial tile after several rounds
+    per = (1 << 13) // n
+    for batch in (1, per - 1, 2 * per, 500 * per + 3):
+        xs, xc = seeded((batch, n), 19, "uniform", dtype)
+        x = to_device(xs, dtype)
+        plan = W.Plan((n,), DT[dtype], W.INVERSE, batch, W.NORM_ORTHO)
+        try:
+            plan.set_pass_variant(0, e, PIPE + 13)
+            guard = torch.zeros((batch + per) * n * x.element_size() // 4 * (1 if dtype == "c32" else 2),
+                                dtype=torch.int32, device="cuda")
+            plan.execute(x.data_ptr(), guard.data_ptr())
+            plan.execute(x.data_ptr(), x.data_ptr())
+            torch.cuda.synchronize()
+        finally:
+            plan.close()
+        words = x.numel() * x.element_size() // 4
+        raw = (torch.view_as_real(x) if dtype == "c32" else x).contiguous().view(-1).view(torch.int32)
+        assert torch.equal(guard[:words], raw) and not guard[words:].any()  # nothing beyond the last pencil
+        ref = oracle.fftn(xc, rank=1, sign=W.INVERSE, norm=oracle.NORM_ORTHO)
+        assert oracle.rel_l2(to_host_c128(x, dtype).reshape(batch, n), ref) < TOL[dtype]
