@@ -223,14 +223,18 @@ int wsfft_execute_host(wsfft_plan plan, const void *host_in, void *host_out,
 int wsfft_destroy(wsfft_plan plan);
 
 /* Plan for `count` independent rank-3 transforms of uneven shapes
- * dims[3*i .. 3*i+2] (each axis a power of two, 32..256), executed by one
- * persistent launch that pulls (instance, superstep, tile) tasks from a
- * queue; a superstep's tiles wait (bounded) until the previous superstep of
- * the same instance is complete.  Section 4.4 (more than one pencil per
- * processor) generalised to one thread block per tile.  Normalisation as
- * wsfft_plan_create (PAPER for WSFFT_C32, ORTHO otherwise).  The launch and
- * its table upload can be captured in a CUDA graph (the upload is skipped
- * when the pointers are unchanged).
+ * dims[3*i .. 3*i+2] (each axis a power of two, 32..256).  16-bit storage,
+ * executes with an instance in place, and plans with a chosen queue variant
+ * (wsfft_plan_set_ragged_variant) run one persistent launch that pulls
+ * (instance, superstep, tile) tasks from a queue; a superstep's tiles wait
+ * (bounded) until the previous superstep of the same instance is complete.
+ * WSFFT_C32 executes out of place run grouped launches instead: one per tile
+ * shape and trip over all instances that have it, two trips per instance
+ * (instances of more than 2^22 elements: three, one after the other).
+ * Section 4.4 (more than one pencil per processor) generalised to one thread
+ * block per tile.  Normalisation as wsfft_plan_create (PAPER for WSFFT_C32,
+ * ORTHO otherwise).  The launches and their table upload can be captured in a
+ * CUDA graph (the upload is skipped when the pointers are unchanged).
  * Errors: INVALID_ARG, INVALID_SIZE, ALLOC, CUDA. */
 int wsfft_plan_create_ragged(wsfft_plan *plan, int count, const int64_t *dims,
                              int dtype, int direction);
@@ -261,8 +265,9 @@ int wsfft_autotune(wsfft_plan plan, wsfft_stream stream);
  * N <= 64, 8 instead of 16 for N >= 128; a tile is always 256 threads);
  * `lag` L puts the y tiles of instance s - L and the x tiles of instance
  * s - 2L after the z tiles of instance s in the queue (1 = the default).
- * Waits for the plan's own work, then rebuilds its tile queue.  Used by
- * wsfft_autotune.  Errors: INVALID_ARG (shape_select outside 0..15, lag
+ * Waits for the plan's own work, then rebuilds its tile queue, which later
+ * executes use whatever their storage type.  Used by wsfft_autotune (which
+ * also times the grouped launches).  Errors: INVALID_ARG (shape_select outside 0..15, lag
  * outside 1..64), UNSUPPORTED (not a ragged plan), ALLOC, CUDA. */
 int wsfft_plan_set_ragged_variant(wsfft_plan plan, int shape_select, int lag);
 

@@ -204,14 +204,20 @@ std::string ragged_key(const Plan &p) {
 }
 
 // the ragged choice is stored in the same line format: mode = lag,
-// variants = [[-1, shape selection, 0]]
+// variants = [[-1, shape selection, 1 for the grouped launches instead of the
+// queue, else 0]]
 int apply_ragged(Plan &p, const Choice &c) {
-    int sel = 0;
+    int sel = 0, grouped = 0;
     for (auto &v : c.variants)
-        if (v[0] == -1) sel = v[1];
-    if (sel < 0 || sel > 15 || c.mode < 1 || c.mode > 64) return WSFFT_ERR_INVALID_ARG;
+        if (v[0] == -1) {
+            sel = v[1];
+            grouped = v[2];
+        }
+    if (sel < 0 || sel > 15 || c.mode < 1 || c.mode > 64 || grouped < 0 || grouped > 1) return WSFFT_ERR_INVALID_ARG;
+    if (grouped && p.dtype != WSFFT_C32) return WSFFT_ERR_INVALID_ARG;
     p.rag_esel = sel;
     p.rag_lag = c.mode;
+    p.rag_grouped = grouped != 0;
     return p.rag_build();
 }
 
@@ -272,14 +278,15 @@ int autotune_ragged(Plan &p, cudaStream_t st) {
         off += (size_t)e * eb;  // a multiple of 16 bytes (axes >= 32)
     }
     const int saved_sel = p.rag_esel, saved_lag = p.rag_lag;
+    const bool saved_grouped = p.rag_grouped;
     Choice best;
     best.mode = saved_lag;
-    best.variants = {{-1, saved_sel, 0}};
+    best.variants = {{-1, saved_sel, saved_grouped ? 1 : 0}};
     double best_us = 1e300;
-    auto consider = [&](int sel, int lag) {
+    auto consider = [&](int sel, int lag, int grouped = 0) {
         Choice c;
         c.mode = lag;
-        c.variants = {{-1, sel, 0}};
+        c.variants = {{-1, sel, grouped}};
         if (apply_ragged(p, c) != WSFFT_SUCCESS) return;
         const double us = time_ragged(p, ip, op, st);
         if (us > 0 && us < best_us) {
@@ -292,6 +299,7 @@ int autotune_ragged(Plan &p, cudaStream_t st) {
         if (present & (1 << k)) consider(best.variants[0][1] ^ (1 << k), best.mode);
     const int sel = best.variants[0][1];
     for (int lag : {2, 4}) consider(sel, lag);
+    consider(0, 1, 1);  // the grouped launches, where the storage type has them
     cudaStreamSynchronize(st);
     cudaFree(in);
     cudaFree(out);
@@ -299,6 +307,7 @@ int autotune_ragged(Plan &p, cudaStream_t st) {
     if (best_us >= 1e300) {
         p.rag_esel = saved_sel;
         p.rag_lag = saved_lag;
+        p.rag_grouped = saved_grouped;
         p.rag_build();
         return WSFFT_ERR_CUDA;
     }

@@ -50,13 +50,17 @@ struct PassArgs {
     // fused tiles (tile_fused.cuh)
     const float2 *tw2;  // stage table of the middle axis
     int64_t elems;      // elements of the launch (slabs: the last tile may be partial)
-    int64_t row;        // elements per row of the last axis
     int64_t ystep;      // elements between the rows of one frequency k1 of the middle axis
     int log_y0;         // log2 of the residue classes of the middle axis' rows
     int log_row;        // log2(row)
     int log_cols;       // log2 of the columns (k1, z) of a transform
     int log_transform;  // log2 of the elements per transform
     int nk1;            // frequencies k1
+    // ragged batches: instance and tile of every tile of the launch, the
+    // instances, and the middle axis' tables by log2(n2) - 5
+    const struct RagRef *refs;
+    const struct RagInst *inst;
+    const float2 *cls[4];
 };
 
 // tile codes at or above this select the complex64 pencil-pair strided

@@ -97,6 +97,20 @@ struct Plan {
     int rag_esel = 0;                  // bit log2(N) - 5: length N uses its second tile shape
     int rag_lag = 1;                   // queue distance (instances) between an instance's supersteps
     int64_t rag_items_cap = 0;
+    // the batch as grouped launches (out of place; rag_grouped: chosen unless a
+    // queue variant is): tile shapes with the tiles of all instances that have
+    // them, and the instances that run on plans of their own
+    struct RagGroup {
+        int kind, b0, b1;      // 0 slab (zb, yb), 1 outer (xb, y0b), 2 strided (points)
+        int64_t ref0, tiles;
+        const float2 *tw, *tw2, *cls[4];
+    };
+    bool rag_grouped = false;
+    std::vector<RagGroup> rag_groups;  // first trips, then last trips
+    size_t rag_first_groups = 0;
+    void *rag_refs = nullptr;          // device RagRef table
+    std::vector<std::pair<int, Plan *>> rag_single;  // instance, its plan
+    std::map<std::vector<int64_t>, Plan *> rag_subplans;  // by shape, owned
     bool withhold = false;         // testing: drop one completion signal
     std::vector<cudaEvent_t> prof_ev;  // 2 per launch slot when profiling
     int prof_used = 0;                 // launch slots recorded since the last read
@@ -121,6 +135,8 @@ struct Plan {
     int build_engine(int64_t n0, int64_t n, bool inv);
     int build_slab(int64_t n0, int64_t n, bool inv);
     int rag_build();                   // ragged plans: instance records and tile queue
+    int rag_build_groups(struct RagInst *inst);  // and the grouped launches
+    int rag_run_grouped(const void *const *in, void *const *out, cudaStream_t st);
     bool slab_runs(int n);             // cluster-fused pass A resident on this device
     int slab_checked[2] = {0, 0};      // per slab edge 256 / 512: 0 unknown, 1 yes, -1 no
     int run(const void *in, void *out, cudaStream_t st);

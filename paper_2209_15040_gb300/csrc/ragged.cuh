@@ -19,18 +19,9 @@
 
 #include "engine.cuh"
 #include "pass_kernels.cuh"
+#include "ragged_desc.h"
 
 namespace wsfft {
-
-struct RagInst {
-    const void *in;
-    void *out;
-    int n[3];          // axis lengths, n[2] contiguous
-    int log_n2, log_n12;
-    int tiles[3];      // tiles of the z, y, x supersteps
-    float scale[3];    // store scale of the z, y, x supersteps
-    int pad;
-};
 
 struct RagItem {
     int flags;     // ITEM_* of engine.cuh; bits 8..9: superstep (0 z, 1 y, 2 x)

@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "pass_kernels.cuh"
+#include "ragged_desc.h"
 #include "tile_desc.h"
 
 namespace wsfft {
@@ -365,7 +366,17 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
     };
     constexpr int EPC = 16 / (int)sizeof(S);  // elements per 16-byte chunk
     auto issue = [&](int64_t tile, int half) {
-        const int64_t base = tile_base(tile);
+        int64_t base, inner = a.inner;
+        const S *from = in;
+        if constexpr (MODE == TILE_STRIDED_RAG) {
+            const RagRef ref = a.refs[tile];
+            const RagInst &I = a.inst[ref.inst];
+            from = static_cast<const S *>(I.out);  // the first trip's output
+            base = (int64_t)ref.tile * G::W;
+            inner = (int64_t)1 << I.log_n12;
+        } else {
+            base = tile_base(tile);
+        }
         if constexpr (MODE == TILE_TRANS) {
             constexpr int CPP = G::N / EPC;  // chunks per pencil
 #pragma unroll
@@ -374,8 +385,8 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         } else {
             constexpr int CPR = G::W / EPC, ROWS = NT / CPR;  // chunks per row, rows per round
             static_assert(CPR <= NT && G::N % ROWS == 0, "whole rounds");
-            const S *p = in + base + (int64_t)(tid / CPR) * a.inner + (tid % CPR) * EPC;
-            const int64_t step = (int64_t)ROWS * a.inner;
+            const S *p = from + base + (int64_t)(tid / CPR) * inner + (tid % CPR) * EPC;
+            const int64_t step = (int64_t)ROWS * inner;
 #pragma unroll
             for (int j = 0; j < G::N / ROWS; ++j) {
                 cp_async16(sm + (tid + j * NT) * 16, p);
@@ -414,8 +425,6 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
     const int slots1 = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid), slots = tile_thread_off<G, TILE_OFF_SLOT, LAST>(tid);
     const int wcol = slots & (G::W - 1), k1 = tile_k_of<G, LAST>(slots);
 
-    const int64_t ostride = MODE == TILE_TRANS ? a.trans_rows : a.inner;
-
     int half = 0;
     int64_t tile = blockIdx.x;
     if (tile < ntiles) issue(tile, 0);
@@ -446,14 +455,26 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         tile_stage<G, LAST, LDG>(v, tw, slots);
         // row k = k1 + Ns r: the last digit r in the registers
         constexpr int Ns = 1 << G::nsbits(LAST), R = 1 << G::gbits(LAST);
-        const int64_t base = tile_base(tile);
-        int64_t ob = base;
+        int64_t ob, ostride = MODE == TILE_TRANS ? a.trans_rows : a.inner;
+        S *o = out;
+        float sx = a.sx, sy = a.sy;
+        if constexpr (MODE == TILE_STRIDED_RAG) {
+            const RagRef ref = a.refs[tile];
+            const RagInst &I = a.inst[ref.inst];
+            ob = (int64_t)ref.tile * G::W;
+            ostride = (int64_t)1 << I.log_n12;
+            o = static_cast<S *>(I.out);
+            sx *= I.last;
+            sy *= I.last;
+        } else {
+            ob = tile_base(tile);
+        }
         if constexpr (MODE == TILE_TRANS) {
             // rows per transform are a multiple of W: a tile's rows share one
-            const int64_t q0 = base / G::N, b = q0 / a.trans_rows;
+            const int64_t q0 = ob / G::N, b = q0 / a.trans_rows;
             ob = b * G::N * a.trans_rows + (q0 - b * a.trans_rows);
         }
-        S *o = out + ob + (int64_t)k1 * ostride + wcol;
+        o += ob + (int64_t)k1 * ostride + wcol;
         const int64_t step = (int64_t)Ns * ostride;
 #pragma unroll
         for (int i = 0; i < 32; i += R) {
@@ -469,8 +490,8 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
                 cpair z = v[i + r];
                 if constexpr (MODE == TILE_STRIDED_TWID)
                     z = cmul(z, cmul(c, ld_cpair(cu + SM::TILE_C / 16 + r * (G::W / 2))));
-                z.re = __fmul2_rn(z.re, f2dup(a.sx));
-                z.im = __fmul2_rn(z.im, f2dup(a.sy));
+                z.re = __fmul2_rn(z.re, f2dup(sx));
+                z.im = __fmul2_rn(z.im, f2dup(sy));
                 SplitPair<S>::store(reinterpret_cast<PT *>(p), z);
                 p += step;
             }

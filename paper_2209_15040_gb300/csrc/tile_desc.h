@@ -11,7 +11,8 @@ namespace wsfft {
 enum {
     TILE_STRIDED = 0,       // strided axis
     TILE_STRIDED_TWID = 1,  // strided axis, four-step twiddle on the store
-    TILE_TRANS = 2          // contiguous axis, transposed store
+    TILE_TRANS = 2,         // contiguous axis, transposed store
+    TILE_STRIDED_RAG = 3    // strided axis, instances of a ragged batch
 };
 
 // Values per thread of the twiddle table a tile kernel's axis of length N
@@ -48,5 +49,11 @@ cudaError_t launch_tile_wide_c16bf(int zb, int rb, const void *in, void *out, co
 cudaError_t launch_tile_outer_c32(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_outer_c16f(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);
 cudaError_t launch_tile_outer_c16bf(int xb, int y0b, const void *in, void *out, const PassArgs &a, cudaStream_t st);
+
+// The same for tiles of several instances of a ragged batch (complex64):
+// a.refs[tile] for `a.tiles` tiles.
+cudaError_t launch_ragged_slab_c32(int zb, int yb, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_ragged_outer_c32(int xb, int y0b, const PassArgs &a, cudaStream_t st);
+cudaError_t launch_ragged_strided_c32(int N, const PassArgs &a, cudaStream_t st);
 
 }  // namespace wsfft

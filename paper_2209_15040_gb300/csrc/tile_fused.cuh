@@ -18,6 +18,7 @@
 // elements).
 #pragma once
 
+#include "ragged_desc.h"
 #include "tile.cuh"
 
 namespace wsfft {
@@ -261,9 +262,9 @@ __device__ __forceinline__ void tile_load(cpair (&v)[32], const S *lbuf, float c
     }
 }
 template <class S>
-__device__ __forceinline__ void tile_store(S *p, cpair z, const PassArgs &a) {
-    z.re = __fmul2_rn(z.re, f2dup(a.sx));
-    z.im = __fmul2_rn(z.im, f2dup(a.sy));
+__device__ __forceinline__ void tile_store(S *p, cpair z, float sx, float sy) {
+    z.re = __fmul2_rn(z.re, f2dup(sx));
+    z.im = __fmul2_rn(z.im, f2dup(sy));
     SplitPair<S>::store(reinterpret_cast<typename SplitPair<S>::T *>(p), z);
 }
 
@@ -278,7 +279,7 @@ __device__ __forceinline__ void tile_store(S *p, cpair z, const PassArgs &a) {
 // WHOLE: tiles of whole slabs (or pencils) of 2^(ZB+YB) < 2^13 elements (the last tile may
 // be partial); otherwise the rows of one residue class of a slab of 2^13
 // << a.log_y0 elements.
-template <class G, class S, bool WHOLE>
+template <class G, class S, bool WHOLE, bool RAG = false>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     tile_slab_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
     using SM = TileFusedSmem<G, S>;
@@ -295,10 +296,20 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int64_t ntiles = a.tiles;
 
-    auto issue = [&](int64_t tile) {
+    auto issue = [&](int64_t t) {
+        int64_t tile = t;
+        const S *from = in;
+        int log_y0 = a.log_y0;
+        if constexpr (RAG) {
+            const RagRef ref = a.refs[t];
+            const RagInst &I = a.inst[ref.inst];
+            tile = ref.tile;
+            from = static_cast<const S *>(I.in);
+            log_y0 = I.log_y0;
+        }
         if constexpr (WHOLE) {
-            const int64_t base = tile << G::TB, left = a.elems - base;
-            const S *src = in + base + tid * EPC;
+            const int64_t base = tile << G::TB, left = RAG ? ELEMS : a.elems - base;
+            const S *src = from + base + tid * EPC;
             if (left >= ELEMS) {
 #pragma unroll
                 for (int j = 0; j < CHUNKS / NT; ++j)
@@ -313,8 +324,9 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
             // slab tile >> log_y0, rows y0, y0 + Y0, ...
             constexpr int CPR = (1 << (G::C2 + 4)) / EPC, ROWS = NT / CPR;  // chunks per row, rows per round
             static_assert(CPR <= NT, "whole rounds");
-            const int64_t rs = a.row << a.log_y0;
-            const S *p = in + ((tile >> a.log_y0) << (G::TB + a.log_y0)) + (tile & ((1 << a.log_y0) - 1)) * a.row +
+            constexpr int64_t row = 1 << (G::C2 + 4);
+            const int64_t rs = row << log_y0;
+            const S *p = from + ((tile >> log_y0) << (G::TB + log_y0)) + (tile & ((1 << log_y0) - 1)) * row +
                          (int64_t)(tid / CPR) * rs + (tid % CPR) * EPC;
             const int64_t step = (int64_t)ROWS * rs;
 #pragma unroll
@@ -354,22 +366,31 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         cp_async_commit();
         tile_gstage<G, LAST, LDG>(v, tw0, tw1, slots2);
-        const int64_t base = tile << G::TB;
-        S *o = out + base + to;
+        int64_t base = tile << G::TB;
+        S *o = out;
+        float sx = a.sx, sy = a.sy;
+        if constexpr (RAG) {
+            const RagRef ref = a.refs[tile];
+            const RagInst &I = a.inst[ref.inst];
+            base = (int64_t)ref.tile << G::TB;
+            o = static_cast<S *>(I.out);
+            sx = sy = I.first;
+        }
+        o += base + to;
         int lim = ELEMS;
-        if constexpr (WHOLE)
+        if constexpr (WHOLE && !RAG)
             if (a.elems - base < ELEMS) lim = (int)(a.elems - base) - to;
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
             const int at = G::place(tile_reg_off<G, TILE_OFF_SLOT, LAST>(r));
-            if (!WHOLE || at < lim) tile_store(o + at, v[r], a);
+            if (!WHOLE || RAG || at < lim) tile_store(o + at, v[r], sx, sy);
         }
     }
 }
 
 // Bound like the strided tiles: complex64 by the memory system (0.35-0.36 ms
 // per 2^27 elements), 16-bit storage by the SM (0.19-0.21).
-template <class G, class S>
+template <class G, class S, bool RAG = false>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     tile_outer_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
     using SM = TileFusedSmem<G, S>;
@@ -390,12 +411,23 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         const int lp = a.log_cols - G::LW;
         return ((tile >> lp) << a.log_transform) + ((tile & (((int64_t)1 << lp) - 1)) << G::LW);
     };
-    auto issue = [&](int64_t tile) {
+    auto issue = [&](int64_t t) {
+        const S *from = in;
+        int64_t base, inner = a.inner;
+        if constexpr (RAG) {
+            const RagRef ref = a.refs[t];
+            const RagInst &I = a.inst[ref.inst];
+            from = static_cast<const S *>(I.out);  // the first trip's output
+            base = (int64_t)ref.tile << G::LW;
+            inner = (int64_t)1 << I.log_n12;
+        } else {
+            base = tile_base(t);
+        }
         // rows of W elements: the n0 rows of a y0, then the next y0
         constexpr int EPC = 16 / (int)sizeof(S), CPR = G::W / EPC, ROWS = NT / CPR, XR = 1 << G::XB;
         static_assert(CPR <= NT && XR % ROWS == 0, "whole rounds");
-        const S *src = in + tile_base(tile) + (int64_t)(tid / CPR) * a.inner + (tid % CPR) * EPC;
-        const int64_t step = (int64_t)ROWS * a.inner;
+        const S *src = from + base + (int64_t)(tid / CPR) * inner + (tid % CPR) * EPC;
+        const int64_t step = (int64_t)ROWS * inner;
 #pragma unroll
         for (int y = 0; y < (1 << G::YB); ++y) {
             const S *p = src + y * a.ystep;
@@ -411,25 +443,40 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     const int slots = tile_thread_off<G, TILE_OFF_SLOT, 1>(tid);
     // x = kx1 + 2^XH kx2, y row k1 + R k0
     constexpr int XS = G::LW + G::XL, XM = (1 << G::XH) - 1, R = 1 << G::XL;
-    const int64_t to = (int64_t)((slots >> XS) & XM) * a.inner + (slots >> (G::TB - G::YB)) * a.ystep +
-                       (slots & (G::W - 1));
-    const int64_t step = a.inner << G::XH;
 
     int64_t tile = blockIdx.x;
     if (tile < ntiles) issue(tile);
     cp_async_commit();
     for (; tile < ntiles; tile += gridDim.x) {
         cpair v[32];
-        const int64_t base = tile_base(tile);
+        int64_t base, inner = a.inner;
+        int log_row = a.log_row, nk1 = a.nk1;
+        const float2 *wy = a.tw_hi;
+        S *o = out;
+        float sx = a.sx, sy = a.sy;
+        if constexpr (RAG) {
+            const RagRef ref = a.refs[tile];
+            const RagInst &I = a.inst[ref.inst];
+            base = (int64_t)ref.tile << G::LW;
+            inner = (int64_t)1 << I.log_n12;
+            log_row = I.log_n2;
+            nk1 = 1 << (G::TB - log_row);
+            wy = log_row == 5 ? a.cls[0] : log_row == 6 ? a.cls[1] : log_row == 7 ? a.cls[2] : a.cls[3];
+            o = static_cast<S *>(I.out);
+            sx *= I.last;
+            sy *= I.last;
+        } else {
+            base = tile_base(tile);
+        }
         cp_async_wait_all();
         __syncthreads();
         tile_load<G, S>(v, lbuf, a.conj_in);
         __syncthreads();
-        const int k1 = (int)(base >> a.log_row) & (a.nk1 - 1);
+        const int k1 = (int)(base >> log_row) & (nk1 - 1);
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
             const int y = i >> G::XH;
-            if (y > 0) v[i] = cmul(v[i], __ldg(&a.tw_hi[(y - 1) * a.nk1 + k1]));
+            if (y > 0) v[i] = cmul(v[i], __ldg(wy + (y - 1) * nk1 + k1));
         }
         tile_gstage<G, 0, LDG>(v, tw0, tw1, 0);
         tile_exchange<G, 0, true>(v, xw, xr);
@@ -438,14 +485,15 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         cp_async_commit();
         tile_gstage<G, 1, LDG>(v, tw0, tw1, slots);
-        S *o = out + base + to;
+        o += base + (int64_t)((slots >> XS) & XM) * inner + (slots >> (G::TB - G::YB)) * a.ystep + (slots & (G::W - 1));
+        const int64_t step = inner << G::XH;
 #pragma unroll
         for (int i = 0; i < 32; i += R) {
             const int sp = tile_reg_off<G, TILE_OFF_SLOT, 1>(i);
-            S *p = o + (int64_t)((sp >> XS) & XM) * a.inner + (sp >> (G::TB - G::YB)) * a.ystep;
+            S *p = o + (int64_t)((sp >> XS) & XM) * inner + (sp >> (G::TB - G::YB)) * a.ystep;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                tile_store(p, v[i + r], a);
+                tile_store(p, v[i + r], sx, sy);
                 p += step;
             }
         }
@@ -539,7 +587,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
             const int sp = tile_reg_off<G, TILE_OFF_SLOT, 2>(r);
-            tile_store(o + (int64_t)(sp >> ZB) * a.inner + kz(sp), v[r], a);
+            tile_store(o + (int64_t)(sp >> ZB) * a.inner + kz(sp), v[r], a.sx, a.sy);
         }
     }
 }

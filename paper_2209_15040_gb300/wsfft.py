@@ -232,7 +232,9 @@ def transpose_outer(in_ptr: int, out_ptr: int, a: int, b: int, c: int, dtype: in
 
 
 class RaggedPlan:
-    """One persistent launch over ``count`` rank-3 transforms of uneven shapes."""
+    """``count`` rank-3 transforms of uneven shapes per execute: grouped launches
+    over all instances of a tile shape (complex64 out of place), otherwise one
+    persistent launch (see wsfft_plan_create_ragged)."""
 
     def __init__(self, shapes, dtype: int = C32, direction: int = FORWARD):
         self.shapes = [tuple(int(v) for v in s) for s in shapes]
