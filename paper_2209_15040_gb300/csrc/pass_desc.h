@@ -61,6 +61,7 @@ struct PassArgs {
     const struct RagRef *refs;
     const struct RagInst *inst;
     const float2 *cls[4];
+    int late;           // wait for the launches before at the end instead of at the start
 };
 
 // tile codes at or above this select the complex64 pencil-pair strided

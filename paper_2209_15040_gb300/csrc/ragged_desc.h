@@ -20,7 +20,7 @@ struct RagInst {
 };
 
 // Grouped launches: the tile of an instance that a launch's tile is.
-struct RagRef {
+struct alignas(8) RagRef {
     int inst, tile;
 };
 

@@ -37,6 +37,31 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *g) {
     const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(g) : "memory");
 }
+// until the grids before this one in the stream are complete
+__device__ __forceinline__ void tile_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A tile of a ragged launch and what its instance says, read from L2: a launch
+// that does not wait at its start (PassArgs::late) must not meet an older line
+// in L1.  The kernels read the next tile's a whole tile ahead: two dependent
+// L2 reads in front of the copies and again of the stores cost 2%.
+struct RagTile {
+    const void *in;
+    void *out;
+    int64_t tile;
+    int log_n2, log_n12, log_y0;
+    float first, last;
+};
+template <class T>
+__device__ __forceinline__ T *ldcg_ptr(T *const *p) {
+    return reinterpret_cast<T *>(__ldcg(reinterpret_cast<const unsigned long long *>(p)));
+}
+__device__ __forceinline__ RagTile rag_tile(const PassArgs &a, int64_t t) {
+    const int2 r = __ldcg(reinterpret_cast<const int2 *>(a.refs) + t);
+    const RagInst *i = a.inst + r.x;
+    return RagTile{ldcg_ptr(&i->in), ldcg_ptr(&i->out), r.y, __ldcg(&i->log_n2), __ldcg(&i->log_n12),
+                   __ldcg(&i->log_y0), __ldcg(&i->first), __ldcg(&i->last)};
+}
+
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
@@ -355,7 +380,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         for (int i = tid; i < G::TABLE; i += NT) st[i] = a.tw[i];
         tw = st;
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (MODE != TILE_STRIDED_RAG || !a.late) tile_grid_wait();
     const int64_t ntiles = a.tiles;
 
     // first element of a tile in `in`
@@ -365,15 +390,14 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         else return ((q >> a.log_inner) * ((int64_t)G::N << a.log_inner)) + (q & (a.inner - 1));
     };
     constexpr int EPC = 16 / (int)sizeof(S);  // elements per 16-byte chunk
+    RagTile rag{}, rag_next{};  // the tile in hand, the one after it
     auto issue = [&](int64_t tile, int half) {
         int64_t base, inner = a.inner;
         const S *from = in;
         if constexpr (MODE == TILE_STRIDED_RAG) {
-            const RagRef ref = a.refs[tile];
-            const RagInst &I = a.inst[ref.inst];
-            from = static_cast<const S *>(I.out);  // the first trip's output
-            base = (int64_t)ref.tile * G::W;
-            inner = (int64_t)1 << I.log_n12;
+            from = static_cast<const S *>(rag_next.out);  // the first trip's output
+            base = rag_next.tile * G::W;
+            inner = (int64_t)1 << rag_next.log_n12;
         } else {
             base = tile_base(tile);
         }
@@ -427,10 +451,16 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
 
     int half = 0;
     int64_t tile = blockIdx.x;
+    if constexpr (MODE == TILE_STRIDED_RAG)
+        if (tile < ntiles) rag_next = rag_tile(a, tile);
     if (tile < ntiles) issue(tile, 0);
     cp_async_commit();
     for (; tile < ntiles; tile += gridDim.x) {
         cpair v[32];
+        if constexpr (MODE == TILE_STRIDED_RAG) {
+            rag = rag_next;
+            if (tile + gridDim.x < ntiles) rag_next = rag_tile(a, tile + gridDim.x);
+        }
         cp_async_wait_all();
         __syncthreads();
 #pragma unroll
@@ -459,13 +489,11 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         S *o = out;
         float sx = a.sx, sy = a.sy;
         if constexpr (MODE == TILE_STRIDED_RAG) {
-            const RagRef ref = a.refs[tile];
-            const RagInst &I = a.inst[ref.inst];
-            ob = (int64_t)ref.tile * G::W;
-            ostride = (int64_t)1 << I.log_n12;
-            o = static_cast<S *>(I.out);
-            sx *= I.last;
-            sy *= I.last;
+            ob = rag.tile * G::W;
+            ostride = (int64_t)1 << rag.log_n12;
+            o = static_cast<S *>(rag.out);
+            sx *= rag.last;
+            sy *= rag.last;
         } else {
             ob = tile_base(tile);
         }
@@ -498,6 +526,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
         }
         half ^= 1;
     }
+    if (MODE == TILE_STRIDED_RAG && a.late) tile_grid_wait();
 }
 
 }  // namespace wsfft

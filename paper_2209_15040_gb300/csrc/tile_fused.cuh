@@ -293,19 +293,18 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     const int tid = threadIdx.x;
     const float2 *tw0, *tw1;
     tile_tables<G, S>(sm, a, tw0, tw1);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!RAG || !a.late) tile_grid_wait();
     const int64_t ntiles = a.tiles;
 
+    RagTile rag{}, rag_next{};  // the tile in hand, the one after it
     auto issue = [&](int64_t t) {
         int64_t tile = t;
         const S *from = in;
         int log_y0 = a.log_y0;
         if constexpr (RAG) {
-            const RagRef ref = a.refs[t];
-            const RagInst &I = a.inst[ref.inst];
-            tile = ref.tile;
-            from = static_cast<const S *>(I.in);
-            log_y0 = I.log_y0;
+            tile = rag_next.tile;
+            from = static_cast<const S *>(rag_next.in);
+            log_y0 = rag_next.log_y0;
         }
         if constexpr (WHOLE) {
             const int64_t base = tile << G::TB, left = RAG ? ELEMS : a.elems - base;
@@ -347,10 +346,16 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     const int to = G::place(slots2);
 
     int64_t tile = blockIdx.x;
+    if constexpr (RAG)
+        if (tile < ntiles) rag_next = rag_tile(a, tile);
     if (tile < ntiles) issue(tile);
     cp_async_commit();
     for (; tile < ntiles; tile += gridDim.x) {
         cpair v[32];
+        if constexpr (RAG) {
+            rag = rag_next;
+            if (tile + gridDim.x < ntiles) rag_next = rag_tile(a, tile + gridDim.x);
+        }
         cp_async_wait_all();
         __syncthreads();
         tile_load<G, S>(v, lbuf, a.conj_in);
@@ -370,11 +375,9 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         S *o = out;
         float sx = a.sx, sy = a.sy;
         if constexpr (RAG) {
-            const RagRef ref = a.refs[tile];
-            const RagInst &I = a.inst[ref.inst];
-            base = (int64_t)ref.tile << G::TB;
-            o = static_cast<S *>(I.out);
-            sx = sy = I.first;
+            base = rag.tile << G::TB;
+            o = static_cast<S *>(rag.out);
+            sx = sy = rag.first;
         }
         o += base + to;
         int lim = ELEMS;
@@ -386,6 +389,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
             if (!WHOLE || RAG || at < lim) tile_store(o + at, v[r], sx, sy);
         }
     }
+    if (RAG && a.late) tile_grid_wait();
 }
 
 // Bound like the strided tiles: complex64 by the memory system (0.35-0.36 ms
@@ -402,7 +406,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     const int tid = threadIdx.x;
     const float2 *tw0, *tw1;
     tile_tables<G, S>(sm, a, tw0, tw1);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!RAG || !a.late) tile_grid_wait();
     const int64_t ntiles = a.tiles;
 
     // columns (k1, z) of a transform: 2^log_cols of them, W per tile
@@ -411,15 +415,14 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         const int lp = a.log_cols - G::LW;
         return ((tile >> lp) << a.log_transform) + ((tile & (((int64_t)1 << lp) - 1)) << G::LW);
     };
+    RagTile rag{}, rag_next{};  // the tile in hand, the one after it
     auto issue = [&](int64_t t) {
         const S *from = in;
         int64_t base, inner = a.inner;
         if constexpr (RAG) {
-            const RagRef ref = a.refs[t];
-            const RagInst &I = a.inst[ref.inst];
-            from = static_cast<const S *>(I.out);  // the first trip's output
-            base = (int64_t)ref.tile << G::LW;
-            inner = (int64_t)1 << I.log_n12;
+            from = static_cast<const S *>(rag_next.out);  // the first trip's output
+            base = rag_next.tile << G::LW;
+            inner = (int64_t)1 << rag_next.log_n12;
         } else {
             base = tile_base(t);
         }
@@ -445,26 +448,30 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     constexpr int XS = G::LW + G::XL, XM = (1 << G::XH) - 1, R = 1 << G::XL;
 
     int64_t tile = blockIdx.x;
+    if constexpr (RAG)
+        if (tile < ntiles) rag_next = rag_tile(a, tile);
     if (tile < ntiles) issue(tile);
     cp_async_commit();
     for (; tile < ntiles; tile += gridDim.x) {
         cpair v[32];
+        if constexpr (RAG) {
+            rag = rag_next;
+            if (tile + gridDim.x < ntiles) rag_next = rag_tile(a, tile + gridDim.x);
+        }
         int64_t base, inner = a.inner;
         int log_row = a.log_row, nk1 = a.nk1;
         const float2 *wy = a.tw_hi;
         S *o = out;
         float sx = a.sx, sy = a.sy;
         if constexpr (RAG) {
-            const RagRef ref = a.refs[tile];
-            const RagInst &I = a.inst[ref.inst];
-            base = (int64_t)ref.tile << G::LW;
-            inner = (int64_t)1 << I.log_n12;
-            log_row = I.log_n2;
+            base = rag.tile << G::LW;
+            inner = (int64_t)1 << rag.log_n12;
+            log_row = rag.log_n2;
             nk1 = 1 << (G::TB - log_row);
             wy = log_row == 5 ? a.cls[0] : log_row == 6 ? a.cls[1] : log_row == 7 ? a.cls[2] : a.cls[3];
-            o = static_cast<S *>(I.out);
-            sx *= I.last;
-            sy *= I.last;
+            o = static_cast<S *>(rag.out);
+            sx *= rag.last;
+            sy *= rag.last;
         } else {
             base = tile_base(tile);
         }
@@ -498,6 +505,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
             }
         }
     }
+    if (RAG && a.late) tile_grid_wait();
 }
 
 // One digit of a strided axis of n points (element stride a.inner, a multiple
@@ -520,7 +528,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     const int tid = threadIdx.x;
     const float2 *tw0, *tw1;
     tile_tables<G, S>(sm, a, tw0, tw1);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    tile_grid_wait();
     const int64_t ntiles = a.tiles;
 
     const int log_m = a.log_inner - ZB;  // rows within the axis' stride

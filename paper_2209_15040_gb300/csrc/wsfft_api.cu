@@ -1582,8 +1582,9 @@ int Plan::run_host_pipelined(const void *hin, void *hout, cudaStream_t st) {
 // tile shape and trip over all of them; the others (more than 2^22 elements,
 // or rows shorter than a tile's) run one after the other on plans of their
 // own.  256 shapes of 32..256 points per axis: 3.95 ms as one queue, whose
-// tiles make three trips at 0.87 of the copy rate, 2.91 ms so (64 shapes 1040
-// and 840 us, 12 shapes 168 both ways, one 20.7 and 10.2).
+// tiles make three trips at 0.87 of the copy rate, 2.90 ms so; 48 shapes
+// 535-749 us and 436-617, 12 shapes 114-253 and 83-238 (half of the elements in
+// instances on plans of their own), 8 shapes 87-152 and 59-148, one 20.8 and 10.4.
 int Plan::rag_build_groups(RagInst *inst) {
     rag_groups.clear();
     rag_single.clear();
@@ -1662,6 +1663,12 @@ int Plan::rag_build_groups(RagInst *inst) {
     return upload(rag_refs, refs.data(), refs.size() * sizeof(RagRef));
 }
 
+// The launches of one trip do not depend on each other: only its first waits
+// at its start for what is before it in the stream, the others at their end.
+// A launch starts once every block of the one before it has let it (after
+// that one's own wait, if it has one), so all of a trip's launches start
+// after what the first waited for; and a launch is complete only when the one
+// before it is, so whatever waits for the last one waits for all.
 int Plan::rag_run_grouped(const void *const *in, void *const *out, cudaStream_t st) {
     auto run_groups = [&](size_t from, size_t to) {
         for (size_t i = from; i < to; ++i) {
@@ -1674,6 +1681,7 @@ int Plan::rag_run_grouped(const void *const *in, void *const *out, cudaStream_t 
             a.tw2 = g.tw2;
             for (int k = 0; k < 4; ++k) a.cls[k] = g.cls[k];
             a.ystep = (int64_t)1 << FUSED_TILE_BITS;
+            a.late = i > from;
             // the inverse conjugates on the first load and on the last store
             a.conj_in = g.kind == 0 && dir == WSFFT_INVERSE ? -1.f : 1.f;
             a.sx = 1.f;
