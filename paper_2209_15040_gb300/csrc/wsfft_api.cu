@@ -614,6 +614,14 @@ void Plan::defer_scale(std::vector<PassSpec> &list) const {
 int Plan::build_fused(const std::vector<int64_t> &d, bool inv) {
     const FusedShape f = fused_tile_rule(d);
     if (!f.use) return WSFFT_SUCCESS;
+    // Below 2^17 elements a block's time for 2^13 elements (about 4 us) is more than
+    // two launches over many small blocks take: one 64 x 64 plane 5.5 us against
+    // 3.1, 32 x 32 x 64 6.3 against 5.1 (2^17 and more: 64^3 7.1 against 9.1, eight
+    // 32^3 6.7 against 11.1).  The smaller tiles of 32 x 32 slabs make up for that
+    // from 2^15 elements up in complex64: 32^3 5.2 us either way, one launch fewer.
+    const int64_t total = elems * batch;
+    if (total < FUSED_SMALL_ELEMS && !(dtype == WSFFT_C32 && f.zb + f.yb == 10 && total >= FUSED_SMALL_ELEMS / 4))
+        return WSFFT_SUCCESS;
     const int r = (int)d.size();
     const int64_t n1 = d[r - 2], n2 = d[r - 1], n0 = r == 3 ? d[0] : 1;
     const int64_t rows = (int64_t)1 << f.yb;

@@ -56,11 +56,15 @@ def _check(dims, batch, dtype, direction, passes):
 @pytest.mark.parametrize("dtype", ["c32", "c16f", "c16bf"])
 @pytest.mark.parametrize("n1,n2", SLABS)
 def test_whole_slabs(dtype, n1, n2):
-    # planes that fill no tile, and a last tile that is partial
-    per = (1 << 13) // (n1 * n2)
-    _check((n1, n2), 1, dtype, W.FORWARD, 1)
-    _check((n1, n2), 3 * per + 1, dtype, W.INVERSE, 1)
-    _check((2, n1, n2), 5, dtype, W.FORWARD, 2)
+    # below 2^17 elements one launch per axis, but for complex64 batches of
+    # 32 x 32 slabs from 2^15 elements up (tiles of 2^11); then tiles of 2^13;
+    # the last tile partial
+    per, small = (1 << 13) // (n1 * n2), n1 * n2 == 1 << 10 and dtype == "c32"
+    _check((n1, n2), 1, dtype, W.FORWARD, 2)
+    _check((n1, n2), 5 * per + 1, dtype, W.INVERSE, 1 if small else 2)
+    _check((n1, n2), 16 * per + 1, dtype, W.INVERSE, 1)
+    _check((2, n1, n2), 2 * per + 1, dtype, W.FORWARD, 2 if small else 3)
+    _check((2, n1, n2), 8 * per + 1, dtype, W.FORWARD, 2)
 
 
 @pytest.mark.parametrize("dtype", ["c32", "c16f", "c16bf"])
