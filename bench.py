@@ -491,9 +491,9 @@ def _ragged_graph_time(plan, ins, outs, dev, stream, reps):
 
 def ragged_leg(W, dev, stream, reps=5):
     """The ragged configuration (256 uneven 3D shapes from seed 4, N(0,1)):
-    one persistent launch replayed from a captured CUDA graph, with the
-    default tile shapes and after wsfft_autotune, vs one plan execute per
-    instance (3 launches each)."""
+    the plan's launches replayed from a captured CUDA graph, as created and
+    after wsfft_autotune, vs one plan execute per instance.  launches_batch
+    counts a large instance's plan as one."""
     from paper_2209_15040_gb300 import inputs
     shapes = inputs.ragged_shapes(256, 4)
     g = torch.Generator(device=dev)
@@ -506,8 +506,8 @@ def ragged_leg(W, dev, stream, reps=5):
     elems = int(sum(int(np.prod(s)) for s in shapes))
     ins, outs = [x.data_ptr() for x in xs], [y.data_ptr() for y in ys]
     plan = W.RaggedPlan(shapes, W.C32, W.FORWARD)
-    # the default tile shapes and lag, then the autotuned choice (tile shape
-    # per axis length, queue lag), each replayed from a captured graph
+    # the default (grouped launches), then the autotuned choice (grouped, or
+    # the queue's tile shape per axis length and lag), each replayed from a captured graph
     t_default = _ragged_graph_time(plan, ins, outs, dev, stream, reps)
     import tempfile
     tune = {}
@@ -518,13 +518,19 @@ def ragged_leg(W, dev, stream, reps=5):
             plan.autotune()
             with open(os.environ["WSFFT_TUNE_CACHE"]) as fh:
                 rec = json.loads(fh.read().strip().splitlines()[-1])
-            tune = {"shape_select": rec["variants"][0][1], "lag": rec["mode"]}
+            tune = {"shape_select": rec["variants"][0][1], "lag": rec["mode"], "grouped": rec["variants"][0][2]}
         finally:
             if prev is None:
                 del os.environ["WSFFT_TUNE_CACHE"]
             else:
                 os.environ["WSFFT_TUNE_CACHE"] = prev
     t_graph = _ragged_graph_time(plan, ins, outs, dev, stream, reps)
+    import ctypes
+    lib, count = W.lib(), ctypes.c_int()
+    lib.wsfft_plan_profile(plan.handle, 256)
+    plan.execute(ins, outs, stream)
+    lib.wsfft_plan_launch_times(plan.handle, None, 0, ctypes.byref(count))
+    lib.wsfft_plan_profile(plan.handle, 0)
     plans = [W.Plan(tuple(int(v) for v in s), W.C32, W.FORWARD, 1) for s in shapes]
     launches = sum(p.passes()[0] for p in plans)
     def per_instance():
@@ -546,7 +552,7 @@ def ragged_leg(W, dev, stream, reps=5):
     return {"instances": len(shapes), "elements": elems, "bytes": elems * 8,
             "persistent_graph_us": round(t_graph, 1), "persistent_graph_default_us": round(t_default, 1),
             "autotuned": tune, "per_instance_us": round(t_inst, 1),
-            "speedup": round(t_inst / t_graph, 3), "launches_persistent": 1,
+            "speedup": round(t_inst / t_graph, 3), "launches_batch": count.value,
             "launches_per_instance": launches,
             "hbm_gbs_3pass_equiv": round(3 * 2 * elems * 8 / (t_graph * 1e-6) / 1e9, 1)}
 
