@@ -104,16 +104,17 @@ class SlabFFT3:
         """Shape of this rank's y-slab (the spectral side)."""
         return (self.dims[0], self.n1l, self.dims[2])
 
-    def _check(self, t: torch.Tensor, shape) -> None:
+    def _checked(self, t: torch.Tensor, shape) -> torch.Tensor:
         want = shape[0] * shape[1] * shape[2]
         if not t.is_contiguous() or _elems(t) != want:
             raise ValueError(f"expected a contiguous tensor of {want} complex elements {shape}")
+        return W.materialized(t)
 
     # -- forward ---------------------------------------------------------------
     def forward_pack(self, x: torch.Tensor) -> torch.Tensor:
         """Steps 1-2: local z and y supersteps, then the regrouping by
         destination rank; returns the send buffer [G][n0/G][n1/G][n2]."""
-        self._check(x, self.slab_shape())
+        x = self._checked(x, self.slab_shape())
         t = torch.empty_like(x)
         self.fwd.slab_2d(x, t)
         send = torch.empty_like(x)
@@ -122,8 +123,7 @@ class SlabFFT3:
 
     def forward_finish(self, recv: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
         """Step 4 on the received y-slab [n0][n1/G][n2]: the x superstep."""
-        self._check(recv, self.spectral_shape())
-        recv = _view(recv, self.spectral_shape())
+        recv = _view(self._checked(recv, self.spectral_shape()), self.spectral_shape())
         out = recv if out is None else out
         self.fwd.axis0(recv, out)
         return out
@@ -135,7 +135,7 @@ class SlabFFT3:
     def inverse_pack(self, y: torch.Tensor) -> torch.Tensor:
         """The x superstep of this rank's y-slab; its rows are already
         grouped by destination (x-slab d is rows d*n0/G ..)."""
-        self._check(y, self.spectral_shape())
+        y = self._checked(y, self.spectral_shape())
         send = torch.empty_like(y)
         self.inv.axis0(y, send)
         return _view(send, self.slab_shape())
@@ -143,8 +143,7 @@ class SlabFFT3:
     def inverse_finish(self, recv: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
         """After the exchange: regroup [G][n0/G][n1/G * n2] into row order
         [n0/G][G][n1/G * n2] = [n0/G][n1][n2], then the y and z supersteps."""
-        self._check(recv, self.slab_shape())
-        recv = _view(recv, self.slab_shape())
+        recv = _view(self._checked(recv, self.slab_shape()), self.slab_shape())
         u = torch.empty_like(recv)
         self.inv.regroup(recv, u, self.world, self.n0l, self.n1l * self.dims[2])
         out = u if out is None else out

@@ -295,6 +295,15 @@ def storage_of(x: torch.Tensor):
     raise TypeError(f"unsupported dtype {x.dtype}")
 
 
+def materialized(x: torch.Tensor) -> torch.Tensor:
+    """`x`, or a copy of it where it is a lazy conjugate or negative view: the
+    library reads the storage, which does not hold those.  contiguous() keeps
+    the views lazy."""
+    if x.is_conj() or x.is_neg():
+        x = x.resolve_conj().resolve_neg()
+    return x
+
+
 _plans: "collections.OrderedDict" = collections.OrderedDict()
 _plans_lock = threading.Lock()
 _plan_cache_size = 32
@@ -358,7 +367,7 @@ def _run(x: torch.Tensor, rank, direction: int, norm, out=None) -> torch.Tensor:
     if norm is None:
         norm = NORM_PAPER if code == C32 else NORM_ORTHO
     norm = NORMS[norm] if isinstance(norm, str) else int(norm)
-    x = x.contiguous()
+    x = materialized(x).contiguous()
     if out is None:
         out = torch.empty_like(x)
     if x.numel() == 0:
@@ -400,7 +409,7 @@ class _FFTN(torch.autograd.Function):
     @staticmethod
     def backward(ctx, g):
         adj = _ADJOINT_NORM[(ctx.direction, ctx.norm)]
-        return _run(g.contiguous(), ctx.rank, -ctx.direction, adj), None, None, None
+        return _run(g, ctx.rank, -ctx.direction, adj), None, None, None
 
 
 def _resolve_norm(x, norm):
