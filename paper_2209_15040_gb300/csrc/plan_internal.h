@@ -9,6 +9,8 @@
 #include <utility>
 #include <vector>
 
+#include "host_roots.h"
+
 namespace wsfft {
 
 struct PassArgs;
@@ -115,6 +117,19 @@ struct Plan {
     std::vector<cudaEvent_t> prof_ev;  // 2 per launch slot when profiling
     int prof_used = 0;                 // launch slots recorded since the last read
 
+    // device memory of the tables; pending: the last bytes of it, not copied yet
+    struct TableBlock {
+        char *device = nullptr;
+        size_t size = 0, used = 0;
+        std::vector<char> pending;
+    };
+    std::vector<TableBlock> table_blocks;
+    RootMemo roots;          // while tables are made
+    Plan *lender = nullptr;  // the plan whose stage tables this one uses (ragged: an instance's own plan)
+    float2 *place_table(const std::vector<float2> &h);
+    template <class Map, class Key>
+    const float2 *remember(Map &map, const Key &key, const std::vector<float2> &h);
+    int flush_tables();
     const float2 *table(int N, int E);
     PassArgs pass_args(const PassSpec &p, int64_t npencils) const;
     const float2 *tc_table(int N);  // tensor-core contiguous superstep (tc_contig.cuh)
@@ -123,12 +138,12 @@ struct Plan {
     std::map<std::pair<int64_t, int>, float2 *> fs_tile_tables;  // per long length and first superstep's length
     const float2 *fourstep_tile_table(int64_t L, int N);
     int build_schedule();
+    int make_schedule();     // its pass list, tables not yet on the device
     int build_fused(const std::vector<int64_t> &d, bool inv);
     using StridedBuilder = std::function<PassSpec(int64_t n, int64_t inner)>;
     int build_wide(const std::vector<int64_t> &d, bool inv, const StridedBuilder &strided);
     void defer_scale(std::vector<PassSpec> &list) const;
     const float2 *wide_table(int zb, int rb);
-    float2 *device_table(const std::vector<float2> &h);
     const float2 *table2(int N, int R0);  // two stages of radix R0 and N/R0
     const float2 *class_table(int n, int classes);  // w_n^(y k), y < classes, k < n/classes
     bool overrides_launchable() const;  // every pass-shape override names an instantiated kernel

@@ -47,48 +47,69 @@
 namespace wsfft {
 
 namespace {
-// cos and sin of 2*pi*m/n in long double
-std::pair<long double, long double> host_cos_sin(int64_t m, int64_t n) {
-    m %= n;
-    if (m < 0) m += n;
-    const int64_t o = (8 * m) / n;      // octant
-    const int64_t rho = 8 * m - o * n;  // position inside the octant, [0, n)
-    const long double q = 0.78539816339744830961566084581987572L;  // pi/4
-    long double c, s;
-    if ((o & 1) == 0) {
-        const long double phi = q * (long double)rho / (long double)n;
-        const long double cp = cosl(phi), sp = sinl(phi);
-        switch (o) {
-            case 0: c = cp; s = sp; break;
-            case 2: c = -sp; s = cp; break;
-            case 4: c = -cp; s = -sp; break;
-            default: c = sp; s = -cp; break;  // 6
-        }
-    } else {
-        const long double phi = q * (long double)(n - rho) / (long double)n;
-        const long double cp = cosl(phi), sp = sinl(phi);
-        switch (o) {
-            case 1: c = sp; s = cp; break;
-            case 3: c = -cp; s = sp; break;
-            case 5: c = -sp; s = -cp; break;
-            default: c = cp; s = -sp; break;  // 7
-        }
-    }
-    return {c, s};
+
+// cos and sin of (pi/4) at/n, 0 <= at <= n
+OctantRoot octant_root(int64_t at, int64_t n) {
+    const long double phi = 0.78539816339744830961566084581987572L * (long double)at / (long double)n;
+    const long double c = cosl(phi), s = sinl(phi);
+    return OctantRoot{(float)c, (float)s, (double)c, (double)s};
 }
+
+// cos and -sin of an angle in octant o, from those of its distance to the
+// octant's axis (odd octants are measured from their upper end)
+template <class T>
+std::pair<T, T> unfold(int o, T c, T s) {
+    switch (o) {
+        case 0: return {c, -s};
+        case 1: return {s, -c};
+        case 2: return {-s, -c};
+        case 3: return {-c, -s};
+        case 4: return {-c, s};
+        case 5: return {-s, c};
+        case 6: return {s, c};
+        default: return {c, s};
+    }
+}
+
+// the octant of 2*pi*m/n and the root of the distance to its axis
+OctantRoot fold(int64_t m, int64_t n, RootMemo *memo, int &octant) {
+    const int log_n = __builtin_ctzll((unsigned long long)n);
+    m &= n - 1;
+    octant = (int)((8 * m) >> log_n);
+    const int64_t rho = (8 * m) & (n - 1);  // position inside the octant, [0, n)
+    const int64_t at = (octant & 1) == 0 ? rho : n - rho;
+    if (!memo) return octant_root(at, n);
+    // at/n is the same float for every n: the factors between them are powers of two
+    if (log_n <= RootMemo::LOG_ORDER) {
+        const int64_t i = (at << (RootMemo::LOG_ORDER - log_n)) >> 3;
+        if (!memo->known[i]) {
+            memo->near[i] = octant_root(at, n);
+            memo->known[i] = true;
+        }
+        return memo->near[i];
+    }
+    const auto found = memo->far.try_emplace(at << (32 - log_n));
+    if (found.second) found.first->second = octant_root(at, n);
+    return found.first->second;
+}
+
 }  // namespace
 
-float2 host_root(int64_t m, int64_t n) {
-    const auto cs = host_cos_sin(m, n);
-    return make_float2((float)cs.first, (float)-cs.second);
+float2 host_root(int64_t m, int64_t n, RootMemo *memo) {
+    int o;
+    const OctantRoot r = fold(m, n, memo, o);
+    const auto cs = unfold(o, r.cf, r.sf);
+    return make_float2(cs.first, cs.second);
 }
 
-std::complex<double> host_root_d(int64_t m, int64_t n) {
-    const auto cs = host_cos_sin(m, n);
-    return {(double)cs.first, (double)-cs.second};
+std::complex<double> host_root_d(int64_t m, int64_t n, RootMemo *memo) {
+    int o;
+    const OctantRoot r = fold(m, n, memo, o);
+    const auto cs = unfold(o, r.cd, r.sd);
+    return {cs.first, cs.second};
 }
 
-int fill_stage_table(float2 *dst, int cap, int N, int E) {
+int fill_stage_table(float2 *dst, int cap, int N, int E, RootMemo *memo) {
     const int size = sched_tw_size(N, E);
     if (size + 1 > cap) return -1;
     const int ns = sched_nstages(N, E);
@@ -96,7 +117,7 @@ int fill_stage_table(float2 *dst, int cap, int N, int E) {
         const int R = sched_radix(N, E, s), Ns = sched_ns_before(N, E, s);
         const int off = sched_tw_offset(N, E, s);
         for (int r = 1; r < R; ++r)
-            for (int k = 0; k < Ns; ++k) dst[off + (r - 1) * Ns + k] = host_root((int64_t)r * k, (int64_t)Ns * R);
+            for (int k = 0; k < Ns; ++k) dst[off + (r - 1) * Ns + k] = host_root((int64_t)r * k, (int64_t)Ns * R, memo);
     }
     dst[size] = make_float2(0.f, 0.f);
     return size + 1;
@@ -118,9 +139,9 @@ int ilog2(int64_t n) {
 
 int64_t elem_bytes(int dtype) { return dtype == WSFFT_C32 ? 8 : 4; }
 
-std::vector<float2> stage_table(int N, int E) {
+std::vector<float2> stage_table(int N, int E, RootMemo *memo) {
     std::vector<float2> t((size_t)sched_tw_size(N, E) + 1);
-    fill_stage_table(t.data(), (int)t.size(), N, E);
+    fill_stage_table(t.data(), (int)t.size(), N, E, memo);
     return t;
 }
 
@@ -412,20 +433,51 @@ bool partial_overlap(const void *a, const void *b, size_t bytes) {
 
 namespace wsfft {
 
+// Device address of a copy of h, which flush_tables() makes: a plan's tables
+// lie in blocks of at least 128 KB that are allocated and filled in one piece
+// (an allocation and a synchronised copy for each table took 25 us, more
+// than its roots).  Null when the memory is not there.
+float2 *Plan::place_table(const std::vector<float2> &h) {
+    const size_t bytes = (h.size() * sizeof(float2) + 255) & ~(size_t)255;
+    if (table_blocks.empty() || table_blocks.back().used + bytes > table_blocks.back().size) {
+        TableBlock b;
+        b.size = std::max(bytes, (size_t)128 * 1024);
+        if (cudaMalloc(&b.device, b.size) != cudaSuccess) return nullptr;
+        table_blocks.push_back(std::move(b));
+    }
+    TableBlock &b = table_blocks.back();
+    float2 *d = reinterpret_cast<float2 *>(b.device + b.used);
+    const char *src = reinterpret_cast<const char *>(h.data());
+    b.pending.insert(b.pending.end(), src, src + h.size() * sizeof(float2));
+    b.pending.resize(b.pending.size() + bytes - h.size() * sizeof(float2));
+    b.used += bytes;
+    return d;
+}
+template <class Map, class Key>
+const float2 *Plan::remember(Map &map, const Key &key, const std::vector<float2> &h) {
+    float2 *d = place_table(h);
+    if (d) map[key] = d;
+    return d;
+}
+// Copy the tables placed since the last call to the device.
+int Plan::flush_tables() {
+    roots = RootMemo();
+    for (auto &b : table_blocks) {
+        if (b.pending.empty()) continue;
+        const int rc = upload(b.device + b.used - b.pending.size(), b.pending.data(), b.pending.size());
+        if (rc != WSFFT_SUCCESS) return rc;
+        b.pending.clear();
+        b.pending.shrink_to_fit();
+    }
+    return WSFFT_SUCCESS;
+}
+
 const float2 *Plan::tc_table(int N) {
     if (N != 512 || dtype == WSFFT_C32) return nullptr;
     auto key = std::make_pair(N, TC_TILE);
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
-    std::vector<float2> h = tc_table_host(dtype);
-    float2 *d = nullptr;
-    if (cudaMalloc(&d, h.size() * sizeof(float2)) != cudaSuccess) return nullptr;
-    if (upload(d, h.data(), h.size() * sizeof(float2)) != WSFFT_SUCCESS) {
-        cudaFree(d);
-        return nullptr;
-    }
-    tables[key] = d;
-    return d;
+    return remember(tables, key, tc_table_host(dtype));
 }
 
 // Four-step inter-superstep twiddles w_L^m, m < L, as two tables: the high
@@ -436,16 +488,9 @@ const float2 *Plan::fourstep_table(int64_t L, int shift) {
     if (it != fs_tables.end()) return it->second;
     const int64_t nh = L >> shift, nl = (int64_t)1 << shift;
     std::vector<float2> h((size_t)(nh + nl));
-    for (int64_t i = 0; i < nh; ++i) h[(size_t)i] = host_root(i << shift, L);
-    for (int64_t j = 0; j < nl; ++j) h[(size_t)(nh + j)] = host_root(j, L);
-    float2 *d = nullptr;
-    if (cudaMalloc(&d, h.size() * sizeof(float2)) != cudaSuccess) return nullptr;
-    if (upload(d, h.data(), h.size() * sizeof(float2)) != WSFFT_SUCCESS) {
-        cudaFree(d);
-        return nullptr;
-    }
-    fs_tables[L] = d;
-    return d;
+    for (int64_t i = 0; i < nh; ++i) h[(size_t)i] = host_root(i << shift, L, &roots);
+    for (int64_t j = 0; j < nl; ++j) h[(size_t)(nh + j)] = host_root(j, L, &roots);
+    return remember(fs_tables, L, h);
 }
 
 // The same twiddles for the pipelined tile kernels' first superstep (length
@@ -462,10 +507,10 @@ const float2 *Plan::fourstep_tile_table(int64_t L, int N) {
     const int Ns = tile_table_E(N), shift = (ilog2(L) + 1) / 2;
     const int64_t low = (int64_t)1 << shift;
     std::vector<std::complex<double>> hi((size_t)(L >> shift)), lo((size_t)low);
-    for (size_t i = 0; i < hi.size(); ++i) hi[i] = host_root_d((int64_t)i << shift, L);
-    for (size_t i = 0; i < lo.size(); ++i) lo[i] = host_root_d((int64_t)i, L);
-    std::vector<float> h;
-    h.reserve((size_t)(2 * n1 * (Ns + N / Ns)));
+    for (size_t i = 0; i < hi.size(); ++i) hi[i] = host_root_d((int64_t)i << shift, L, &roots);
+    for (size_t i = 0; i < lo.size(); ++i) lo[i] = host_root_d((int64_t)i, L, &roots);
+    std::vector<float2> h;
+    h.reserve((size_t)(n1 * (Ns + N / Ns)));
     auto rows = [&](int count, int64_t step) {  // w_L^(step q j), j < count
         for (int j = 0; j < count; ++j)
             for (int64_t q = 0; q < n1; q += 2) {
@@ -474,76 +519,55 @@ const float2 *Plan::fourstep_tile_table(int64_t L, int N) {
                     const int64_t m = (step * (q + i) * j) & (L - 1);
                     w[i] = hi[(size_t)(m >> shift)] * lo[(size_t)(m & (low - 1))];
                 }
-                for (double v : {w[0].real(), w[1].real(), w[0].imag(), w[1].imag()}) h.push_back((float)v);
+                h.push_back(make_float2((float)w[0].real(), (float)w[1].real()));
+                h.push_back(make_float2((float)w[0].imag(), (float)w[1].imag()));
             }
     };
     rows(Ns, 1);
     rows(N / Ns, Ns);
-    float2 *d = nullptr;
-    if (cudaMalloc(&d, h.size() * sizeof(float)) != cudaSuccess) return nullptr;
-    if (upload(d, h.data(), h.size() * sizeof(float)) != WSFFT_SUCCESS) {
-        cudaFree(d);
-        return nullptr;
-    }
-    fs_tile_tables[key] = d;
-    return d;
+    return remember(fs_tile_tables, key, h);
 }
 
 const float2 *Plan::table(int N, int E) {
+    if (lender) return lender->table(N, E);
     auto key = std::make_pair(N, E);
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
-    std::vector<float2> h = stage_table(N, E);
-    float2 *d = nullptr;
-    if (cudaMalloc(&d, h.size() * sizeof(float2)) != cudaSuccess) return nullptr;
-    if (upload(d, h.data(), h.size() * sizeof(float2)) != WSFFT_SUCCESS) {
-        cudaFree(d);
-        return nullptr;
-    }
-    tables[key] = d;
-    return d;
-}
-
-// A device copy of a host table, owned by the caller's map (null on failure).
-float2 *Plan::device_table(const std::vector<float2> &h) {
-    float2 *d = nullptr;
-    if (cudaMalloc(&d, h.size() * sizeof(float2)) != cudaSuccess) return nullptr;
-    if (upload(d, h.data(), h.size() * sizeof(float2)) != WSFFT_SUCCESS) {
-        cudaFree(d);
-        return nullptr;
-    }
-    return d;
+    return remember(tables, key, stage_table(N, E, &roots));
 }
 
 // Twiddles of a two-stage pencil, radix R0 then N/R0: w_N^(r k) at
 // (r-1)*R0 + k, r < N/R0, k < R0.
 const float2 *Plan::table2(int N, int R0) {
+    if (lender) return lender->table2(N, R0);
     const auto key = std::make_pair(N, 1000 + R0);
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
     std::vector<float2> h;
     for (int r = 1; r < N / R0; ++r)
-        for (int k = 0; k < R0; ++k) h.push_back(host_root((int64_t)r * k, N));
+        for (int k = 0; k < R0; ++k) h.push_back(host_root((int64_t)r * k, N, &roots));
     h.push_back(make_float2(0.f, 0.f));
-    return tables[key] = device_table(h);
+    return remember(tables, key, h);
 }
 
 // Twiddles between the two parts of a split axis of n points: w_n^(y k) at
 // (y-1)*(n/classes) + k for the residue classes y.
 const float2 *Plan::class_table(int n, int classes) {
+    if (lender) return lender->class_table(n, classes);
     const auto key = std::make_pair(n, 2000 + classes);
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
     std::vector<float2> h;
     for (int y = 1; y < classes; ++y)
-        for (int k = 0; k < n / classes; ++k) h.push_back(host_root((int64_t)y * k, n));
+        for (int k = 0; k < n / classes; ++k) h.push_back(host_root((int64_t)y * k, n, &roots));
     h.push_back(make_float2(0.f, 0.f));
-    return tables[key] = device_table(h);
+    return remember(tables, key, h);
 }
 
 // Stage twiddles of the 2^zb points of a wide tile (TileWide): radices
 // 2^(5-rb), 32 and the rest.
 const float2 *Plan::wide_table(int zb, int rb) {
+    if (lender) return lender->wide_table(zb, rb);
     const auto key = std::make_pair(1 << zb, 3000 + rb);
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
@@ -551,10 +575,10 @@ const float2 *Plan::wide_table(int zb, int rb) {
     int64_t ns = (int64_t)1 << (5 - rb);
     for (int R : {32, (1 << zb) / (32 << (5 - rb))}) {
         for (int r = 1; r < R; ++r)
-            for (int64_t k = 0; k < ns; ++k) h.push_back(host_root(r * k, ns * R));
+            for (int64_t k = 0; k < ns; ++k) h.push_back(host_root(r * k, ns * R, &roots));
         ns *= R;
     }
-    return tables[key] = device_table(h);
+    return remember(tables, key, h);
 }
 
 // Schedule with one digit of a long strided axis in the trip of the last
@@ -884,6 +908,12 @@ int Plan::build_slab(int64_t n0, int64_t n, bool inv) {
 
 // (Re)build the pass list from shape, direction and normalisation.
 int Plan::build_schedule() {
+    const int rc = make_schedule();
+    const int copied = flush_tables();  // also after a failure: the tables made so far are remembered
+    return rc != WSFFT_SUCCESS ? rc : copied;
+}
+
+int Plan::make_schedule() {
     passes.clear();
     fused.clear();
     fused_in_place = false;
@@ -1607,6 +1637,7 @@ int Plan::rag_build_groups(RagInst *inst) {
                 sub = new (std::nothrow) Plan();
                 if (!sub) return WSFFT_ERR_ALLOC;
                 sub->device = device;
+                sub->lender = this;
                 sub->sm_count = sub->eng_grid = sm_count;
                 sub->rank = 3;
                 sub->elems = 1;
@@ -1746,21 +1777,25 @@ int Plan::rag_build() {
     }
     {
         const int rc = rag_build_groups(inst.data());
+        const int copied = flush_tables();
         if (rc != WSFFT_SUCCESS) return rc;
+        if (copied != WSFFT_SUCCESS) return copied;
     }
     const int L = rag_lag;
-    std::vector<RagItem> items;
+    size_t nitems = 0;
+    for (const RagInst &I : inst) nitems += (size_t)I.tiles[0] + I.tiles[1] + I.tiles[2];
+    if (nitems > (size_t)0x7fffffff) return WSFFT_ERR_UNSUPPORTED;
+    std::vector<RagItem> items(nitems);
+    RagItem *item = items.data();
+    auto add = [&](int s, int step, int flags) {
+        if (s < 0 || s >= count) return;
+        for (int t = 0; t < inst[s].tiles[step]; ++t) *item++ = RagItem{flags | (step << 8), s, t, 0};
+    };
     for (int s = 0; s < count + 2 * L; ++s) {
-        if (s < count)
-            for (int t = 0; t < inst[s].tiles[0]; ++t) items.push_back(RagItem{ITEM_SIGNAL | (0 << 8), s, t, 0});
-        if (s - L >= 0 && s - L < count)
-            for (int t = 0; t < inst[s - L].tiles[1]; ++t)
-                items.push_back(RagItem{ITEM_STRIDED | ITEM_WAIT | ITEM_SIGNAL | (1 << 8), s - L, t, 0});
-        if (s - 2 * L >= 0 && s - 2 * L < count)
-            for (int t = 0; t < inst[s - 2 * L].tiles[2]; ++t)
-                items.push_back(RagItem{ITEM_STRIDED | ITEM_WAIT | (2 << 8), s - 2 * L, t, 0});
+        add(s, 0, ITEM_SIGNAL);
+        add(s - L, 1, ITEM_STRIDED | ITEM_WAIT | ITEM_SIGNAL);
+        add(s - 2 * L, 2, ITEM_STRIDED | ITEM_WAIT);
     }
-    if (items.size() > (size_t)0x7fffffff) return WSFFT_ERR_UNSUPPORTED;
     const size_t ib = items.size() * sizeof(RagItem), nb = inst.size() * sizeof(RagInst);
     if (items.size() > (size_t)rag_items_cap) {
         if (rag_items) cudaFree(rag_items);
@@ -1859,9 +1894,7 @@ Plan::~Plan() {
     if (rag_copied) cudaEventDestroy(rag_copied);
     if (d_items) cudaFree(d_items);
     if (d_ctr) cudaFree(d_ctr);
-    for (auto &kv : tables) cudaFree(kv.second);
-    for (auto &kv : fs_tables) cudaFree(kv.second);
-    for (auto &kv : fs_tile_tables) cudaFree(kv.second);
+    for (auto &b : table_blocks) cudaFree(b.device);
     if (work) cudaFree(work);
     if (host_buf) cudaFree(host_buf);
     for (auto e : pipe_ev)
