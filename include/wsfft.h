@@ -248,9 +248,12 @@ int wsfft_execute_ragged(wsfft_plan plan, const void *const *in, void *const *ou
 /* Time the kernel variants that apply to this plan on `stream` (with
  * temporary buffers) and keep the fastest; results are cached in the JSON
  * file named by WSFFT_TUNE_CACHE (if set), keyed by device name, SM count,
- * shape, batch, dtype, direction, normalisation and spectral layout.  For a
- * ragged plan the candidates are the tile shape of each axis length that
- * occurs and the queue lag (wsfft_plan_set_ragged_variant), the key holds
+ * the generation of the library's schedules (a choice timed against other
+ * schedules is not read), shape, batch, dtype, direction, normalisation and
+ * spectral layout.  For a ragged plan the candidates are the tile shape of
+ * each axis length that occurs and the queue lag
+ * (wsfft_plan_set_ragged_variant), then, for WSFFT_C32, the grouped launches
+ * (the fastest queue stays for executes with an instance in place); the key holds
  * the sorted multiset of instance shapes, and a ragged plan created later
  * with the same key takes the cached choice.  A cached entry that does not
  * describe a schedule this build can launch (an unknown schedule, values out
