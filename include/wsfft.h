@@ -269,9 +269,11 @@ int wsfft_autotune(wsfft_plan plan, wsfft_stream stream);
  * `lag` L puts the y tiles of instance s - L and the x tiles of instance
  * s - 2L after the z tiles of instance s in the queue (1 = the default).
  * Waits for the plan's own work, then rebuilds its tile queue, which later
- * executes use whatever their storage type.  Used by wsfft_autotune (which
- * also times the grouped launches).  Errors: INVALID_ARG (shape_select outside 0..15, lag
- * outside 1..64), UNSUPPORTED (not a ragged plan), ALLOC, CUDA. */
+ * executes use whatever their storage type; shape_select 0 with lag 1, the
+ * values of a new plan, also bring back the grouped launches that a new
+ * WSFFT_C32 plan uses out of place.
+ * Errors: INVALID_ARG (shape_select outside 0..15, lag outside 1..64),
+ * UNSUPPORTED (not a ragged plan), ALLOC, CUDA. */
 int wsfft_plan_set_ragged_variant(wsfft_plan plan, int shape_select, int lag);
 
 /* Choose the kernel shape of pass `pass` (0-based, in launch order) of this

@@ -2281,7 +2281,8 @@ int wsfft_plan_set_ragged_variant(wsfft_plan plan, int shape_select, int lag) {
     const bool old_grouped = p->rag_grouped;
     p->rag_esel = shape_select;
     p->rag_lag = lag;
-    p->rag_grouped = false;  // a chosen queue variant is what runs
+    // a chosen queue variant is what runs; the values of a new plan choose what that runs
+    p->rag_grouped = p->dtype == WSFFT_C32 && shape_select == 0 && lag == 1;
     const int rc = p->rag_build();
     if (rc != WSFFT_SUCCESS) {
         p->rag_esel = old_sel;
