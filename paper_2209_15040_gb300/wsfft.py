@@ -105,10 +105,18 @@ def _check(rc: int, what: str) -> None:
         raise WsfftError(rc, what)
 
 
+# Internals of torch that shorten the host path; None where a version lacks one.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_functorch_active = getattr(torch._C, "_are_functorch_transforms_active", None)
+_forward_level = (lambda: forward_ad._current_level) if hasattr(forward_ad, "_current_level") else None
+
+
 def _stream_handle(stream=None) -> int:
     if stream is None:
-        # the handle without a torch.cuda.Stream object around it (0.4 against 2.9 us)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if _raw_stream is not None:
+            # the handle without a torch.cuda.Stream object around it (0.4 against 2.9 us)
+            return _raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -423,9 +431,11 @@ def _transform(x, rank, direction, norm):
     # autograd node, which costs more host time than the launches of a small
     # transform (12 of 33 us per call at 8^3).  Everything else -- gradients,
     # forward-mode levels (no jvp: refused), functorch transforms (no vmap
-    # rule: refused), tracing, tensor subclasses -- goes through the Function.
+    # rule: refused), tracing, tensor subclasses -- goes through the Function, and
+    # so does every call where torch cannot be asked about them.
     if (type(x) is torch.Tensor and not (x.requires_grad and torch.is_grad_enabled())
-            and forward_ad._current_level < 0 and not torch._C._are_functorch_transforms_active()
+            and _forward_level is not None and _forward_level() < 0
+            and _functorch_active is not None and not _functorch_active()
             and not torch.jit.is_tracing()):
         return _run(x, rank, direction, norm)
     return _FFTN.apply(x, rank, direction, norm)
