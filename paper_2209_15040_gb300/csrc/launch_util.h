@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace wsfft {
 
 // Launch with programmatic stream serialization (see pdl_enter): the kernel
@@ -32,11 +34,15 @@ cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), unsigned grid, unsign
 // once per device; threads that race store the same value.
 inline int device_sms() {
     constexpr int kMaxDev = 64;
-    static int sms[kMaxDev] = {};
-    int dev = 0, n = 0;
+    static std::atomic<int> sms[kMaxDev];
+    int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return 0;
-    if (sms[dev] == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) sms[dev] = n;
-    return sms[dev];
+    int n = sms[dev].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+        sms[dev].store(n, std::memory_order_relaxed);
+    }
+    return n;
 }
 
 }  // namespace wsfft
