@@ -13,7 +13,7 @@
 
 namespace wsfft {
 
-struct PassArgs;
+struct TileArgs;
 
 enum { SRC_IN = 0, SRC_OUT = 1, SRC_WORK = 2 };
 enum { DST_OUT = 0, DST_WORK = 1 };
@@ -131,7 +131,7 @@ struct Plan {
     const float2 *remember(Map &map, const Key &key, const std::vector<float2> &h);
     int flush_tables();
     const float2 *table(int N, int E);
-    PassArgs pass_args(const PassSpec &p, int64_t npencils) const;
+    TileArgs pass_args(const PassSpec &p, int64_t npencils) const;
     const float2 *tc_table(int N);  // tensor-core contiguous superstep (tc_contig.cuh)
     std::map<int64_t, float2 *> fs_tables;        // four-step twiddle tables per long length
     const float2 *fourstep_table(int64_t L, int shift);

@@ -10,7 +10,7 @@ namespace wsfft {
 namespace {
 
 template <class SM, class K>
-cudaError_t launch_grouped(K kern, unsigned threads, const PassArgs &a, cudaStream_t st) {
+cudaError_t launch_grouped(K kern, unsigned threads, const TileArgs &a, cudaStream_t st) {
     const cudaError_t attr = set_smem_attr(reinterpret_cast<const void *>(kern), SM::BYTES);
     if (attr != cudaSuccess) return attr;
     if (a.tiles <= 0) return cudaSuccess;
@@ -22,7 +22,7 @@ cudaError_t launch_grouped(K kern, unsigned threads, const PassArgs &a, cudaStre
 
 }  // namespace
 
-cudaError_t launch_ragged_outer_c32(int xb, int y0b, const PassArgs &a, cudaStream_t st) {
+cudaError_t launch_ragged_outer_c32(int xb, int y0b, const TileArgs &a, cudaStream_t st) {
 #define WSFFT_OUTER(x, y)                                                                                   \
     if (xb == x && y0b == y) {                                                                              \
         using G = TileOuter<FUSED_TILE_BITS, x, y>;                                                         \
@@ -41,7 +41,7 @@ cudaError_t launch_ragged_outer_c32(int xb, int y0b, const PassArgs &a, cudaStre
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_ragged_strided_c32(int N, const PassArgs &a, cudaStream_t st) {
+cudaError_t launch_ragged_strided_c32(int N, const TileArgs &a, cudaStream_t st) {
 #define WSFFT_STRIDED(n, b)                                                                                   \
     if (N == n) {                                                                                             \
         using G = TileStrided<FUSED_TILE_BITS, b>;                                                            \

@@ -10,7 +10,7 @@ namespace wsfft {
 namespace {
 
 template <class SM, class K>
-cudaError_t launch_grouped(K kern, unsigned threads, const PassArgs &a, cudaStream_t st) {
+cudaError_t launch_grouped(K kern, unsigned threads, const TileArgs &a, cudaStream_t st) {
     const cudaError_t attr = set_smem_attr(reinterpret_cast<const void *>(kern), SM::BYTES);
     if (attr != cudaSuccess) return attr;
     if (a.tiles <= 0) return cudaSuccess;
@@ -22,7 +22,7 @@ cudaError_t launch_grouped(K kern, unsigned threads, const PassArgs &a, cudaStre
 
 }  // namespace
 
-cudaError_t launch_ragged_slab_c32(int zb, int yb, const PassArgs &a, cudaStream_t st) {
+cudaError_t launch_ragged_slab_c32(int zb, int yb, const TileArgs &a, cudaStream_t st) {
 #define WSFFT_SLAB(z, y)                                                                     \
     if (zb == z && yb == y) {                                                                \
         using G = TileSlab<FUSED_TILE_BITS, z, y>;                                           \

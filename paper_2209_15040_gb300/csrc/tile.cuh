@@ -41,7 +41,7 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *g) {
 __device__ __forceinline__ void tile_grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // A tile of a ragged launch and what its instance says, read from L2: a launch
-// that does not wait at its start (PassArgs::late) must not meet an older line
+// that does not wait at its start (TileArgs::late) must not meet an older line
 // in L1.  The kernels read the next tile's a whole tile ahead: two dependent
 // L2 reads in front of the copies and again of the stores cost 2%.
 struct RagTile {
@@ -55,7 +55,7 @@ template <class T>
 __device__ __forceinline__ T *ldcg_ptr(T *const *p) {
     return reinterpret_cast<T *>(__ldcg(reinterpret_cast<const unsigned long long *>(p)));
 }
-__device__ __forceinline__ RagTile rag_tile(const PassArgs &a, int64_t t) {
+__device__ __forceinline__ RagTile rag_tile(const TileArgs &a, int64_t t) {
     const int2 r = __ldcg(reinterpret_cast<const int2 *>(a.refs) + t);
     const RagInst *i = a.inst + r.x;
     return RagTile{ldcg_ptr(&i->in), ldcg_ptr(&i->out), r.y, __ldcg(&i->log_n2), __ldcg(&i->log_n12),
@@ -364,7 +364,7 @@ struct TileSmem {
 // 0.51, 16-bit 512 points 0.214 against 0.305.
 template <class G, class S, int MODE>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileSmem<G, S, MODE>::CTAS)
-    tile_axis_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
+    tile_axis_kernel(const S *__restrict__ in, S *__restrict__ out, TileArgs a) {
     using SM = TileSmem<G, S, MODE>;
     using PT = typename SplitPair<S>::T;
     constexpr int NT = 1 << (G::TB - 6);

@@ -237,7 +237,7 @@ struct TileFusedSmem {
 
 // The stage tables a kernel reads: in shared memory for 16-bit storage.
 template <class G, class S>
-__device__ __forceinline__ void tile_tables(char *sm, const PassArgs &a, const float2 *&tw0, const float2 *&tw1) {
+__device__ __forceinline__ void tile_tables(char *sm, const TileArgs &a, const float2 *&tw0, const float2 *&tw1) {
     using SM = TileFusedSmem<G, S>;
     tw0 = a.tw;
     tw1 = a.tw2;
@@ -281,7 +281,7 @@ __device__ __forceinline__ void tile_store(S *p, cpair z, float sx, float sy) {
 // << a.log_y0 elements.
 template <class G, class S, bool WHOLE, bool RAG = false>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
-    tile_slab_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
+    tile_slab_kernel(const S *__restrict__ in, S *__restrict__ out, TileArgs a) {
     using SM = TileFusedSmem<G, S>;
     constexpr int NT = 1 << (G::TB - 6), ELEMS = 1 << G::TB;
     constexpr int EPC = 16 / (int)sizeof(S), CHUNKS = ELEMS / EPC;  // elements per 16-byte chunk, chunks per tile
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
 // per 2^27 elements), 16-bit storage by the SM (0.19-0.21).
 template <class G, class S, bool RAG = false>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
-    tile_outer_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
+    tile_outer_kernel(const S *__restrict__ in, S *__restrict__ out, TileArgs a) {
     using SM = TileFusedSmem<G, S>;
     constexpr int NT = 1 << (G::TB - 6);
     constexpr bool LDG = !SM::SHARED_TW;
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
 // tiles of 2^14 elements: 0.485 and 0.37.
 template <class G, class S>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
-    tile_wide_kernel(const S *__restrict__ in, S *__restrict__ out, PassArgs a) {
+    tile_wide_kernel(const S *__restrict__ in, S *__restrict__ out, TileArgs a) {
     using SM = TileFusedSmem<G, S>;
     constexpr int NT = 1 << (G::TB - 6), ZB = G::TB - G::RB;
     constexpr bool LDG = !SM::SHARED_TW;

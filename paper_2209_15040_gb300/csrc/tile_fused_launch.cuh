@@ -13,7 +13,7 @@ namespace wsfft {
 namespace {
 
 template <class G, class K>
-cudaError_t launch_fused(K kern, const void *in, void *out, const PassArgs &a, cudaStream_t st) {
+cudaError_t launch_fused(K kern, const void *in, void *out, const TileArgs &a, cudaStream_t st) {
     using S = WSFFT_STORE;
     using SM = TileFusedSmem<G, S>;
     const cudaError_t attr = set_smem_attr(reinterpret_cast<const void *>(kern), SM::BYTES);
@@ -29,9 +29,9 @@ cudaError_t launch_fused(K kern, const void *in, void *out, const PassArgs &a, c
 }  // namespace
 
 #ifdef WSFFT_SLAB_TILE_NAME
-cudaError_t WSFFT_SLAB_TILE_NAME(int zb, int yb, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
+cudaError_t WSFFT_SLAB_TILE_NAME(int zb, int yb, const void *in, void *out, const TileArgs &arg, cudaStream_t st) {
     using S = WSFFT_STORE;
-    PassArgs a = arg;
+    TileArgs a = arg;
     // Few tiles (complex64 slabs of 2^10): a quarter of a tile's elements per
     // block, one warp each; loads, exchanges and stores take a quarter of the
     // time of one block of four.  32^3: 5.21 us captured and 5.65 in a loop of
@@ -63,9 +63,9 @@ cudaError_t WSFFT_SLAB_TILE_NAME(int zb, int yb, const void *in, void *out, cons
 #endif
 
 #ifdef WSFFT_CONTIG_TILE_NAME
-cudaError_t WSFFT_CONTIG_TILE_NAME(int N, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
+cudaError_t WSFFT_CONTIG_TILE_NAME(int N, const void *in, void *out, const TileArgs &arg, cudaStream_t st) {
     using S = WSFFT_STORE;
-    PassArgs a = arg;
+    TileArgs a = arg;
     a.elems = a.npencils * N;
     a.tiles = (a.elems + (1 << FUSED_TILE_BITS) - 1) >> FUSED_TILE_BITS;
 #define WSFFT_CONTIG(n, b)                                                                                          \
@@ -81,9 +81,9 @@ cudaError_t WSFFT_CONTIG_TILE_NAME(int N, const void *in, void *out, const PassA
 #endif
 
 #ifdef WSFFT_WIDE_TILE_NAME
-cudaError_t WSFFT_WIDE_TILE_NAME(int zb, int rb, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
+cudaError_t WSFFT_WIDE_TILE_NAME(int zb, int rb, const void *in, void *out, const TileArgs &arg, cudaStream_t st) {
     using S = WSFFT_STORE;
-    PassArgs a = arg;
+    TileArgs a = arg;
     a.tiles = a.elems >> (zb + rb);
 #define WSFFT_WIDE(b, z) \
     if (zb == z && rb == b - z) return launch_fused<TileWide<b, z>>(tile_wide_kernel<TileWide<b, z>, S>, in, out, a, st);
@@ -98,9 +98,9 @@ cudaError_t WSFFT_WIDE_TILE_NAME(int zb, int rb, const void *in, void *out, cons
 #endif
 
 #ifdef WSFFT_OUTER_TILE_NAME
-cudaError_t WSFFT_OUTER_TILE_NAME(int xb, int y0b, const void *in, void *out, const PassArgs &arg, cudaStream_t st) {
+cudaError_t WSFFT_OUTER_TILE_NAME(int xb, int y0b, const void *in, void *out, const TileArgs &arg, cudaStream_t st) {
     using S = WSFFT_STORE;
-    PassArgs a = arg;
+    TileArgs a = arg;
     a.tiles = a.elems >> FUSED_TILE_BITS;
 #define WSFFT_OUTER(x, y)                                                                                            \
     if (xb == x && y0b == y)                                                                                         \

@@ -16,7 +16,7 @@ namespace {
 // Persistent launch: as many blocks as are resident at once, each taking
 // every grid-size-th tile.  Whole tiles of adjacent pencils only.
 template <int TB, int NB, int MODE>
-cudaError_t launch_tile_axis(const void *in, void *out, PassArgs a, cudaStream_t st) {
+cudaError_t launch_tile_axis(const void *in, void *out, TileArgs a, cudaStream_t st) {
     using S = WSFFT_STORE;
     using G = std::conditional_t<MODE == TILE_TRANS, TileTrans<TB, NB, (int)sizeof(S)>, TileStrided<TB, NB>>;
     using SM = TileSmem<G, S, MODE>;
@@ -36,7 +36,7 @@ cudaError_t launch_tile_axis(const void *in, void *out, PassArgs a, cudaStream_t
 
 }  // namespace
 
-cudaError_t WSFFT_TILE_NAME(int mode, int N, int tb, const void *in, void *out, const PassArgs &a, cudaStream_t st) {
+cudaError_t WSFFT_TILE_NAME(int mode, int N, int tb, const void *in, void *out, const TileArgs &a, cudaStream_t st) {
     constexpr bool half = sizeof(WSFFT_STORE) == 4;
 #define WSFFT_TILE(m, n, b, nb) \
     if (mode == m && N == n && tb == b) return launch_tile_axis<b, nb, m>(in, out, a, st);

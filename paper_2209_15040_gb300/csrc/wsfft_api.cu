@@ -226,7 +226,7 @@ cudaError_t launch_slab(int dtype, int n, const void *in, void *out, int64_t nsl
     }
 }
 
-cudaError_t launch_tile(int dtype, int mode, int N, int tb, const void *in, void *out, const PassArgs &a,
+cudaError_t launch_tile(int dtype, int mode, int N, int tb, const void *in, void *out, const TileArgs &a,
                         cudaStream_t st) {
     switch (dtype) {
         case WSFFT_C32: return launch_tile_c32(mode, N, tb, in, out, a, st);
@@ -235,9 +235,9 @@ cudaError_t launch_tile(int dtype, int mode, int N, int tb, const void *in, void
     }
 }
 
-cudaError_t launch_fused(int dtype, const PassSpec &p, const void *in, void *out, const PassArgs &a,
+cudaError_t launch_fused(int dtype, const PassSpec &p, const void *in, void *out, const TileArgs &a,
                          cudaStream_t st) {
-    using Fn = cudaError_t (*)(int, int, const void *, void *, const PassArgs &, cudaStream_t);
+    using Fn = cudaError_t (*)(int, int, const void *, void *, const TileArgs &, cudaStream_t);
     static constexpr Fn slab[3] = {launch_tile_slab_c32, launch_tile_slab_c16f, launch_tile_slab_c16bf};
     static constexpr Fn outer[3] = {launch_tile_outer_c32, launch_tile_outer_c16f, launch_tile_outer_c16bf};
     static constexpr Fn wide[3] = {launch_tile_wide_c32, launch_tile_wide_c16f, launch_tile_wide_c16bf};
@@ -245,7 +245,7 @@ cudaError_t launch_fused(int dtype, const PassSpec &p, const void *in, void *out
     return (p.kind == PASS_TILE_SLAB ? slab : wide)[dtype](p.zb, p.yb, in, out, a, st);
 }
 
-cudaError_t launch(int dtype, const PassSpec &p, const void *in, void *out, const PassArgs &a,
+cudaError_t launch(int dtype, const PassSpec &p, const void *in, void *out, const TileArgs &a,
                    cudaStream_t st) {
     if (p.kind == PASS_TILE_SLAB || p.kind == PASS_TILE_OUTER || p.kind == PASS_TILE_WIDE)
         return launch_fused(dtype, p, in, out, a, st);
@@ -1363,7 +1363,7 @@ bool Plan::overrides_launchable() const {
         if (kv.first < 0 || kv.first >= (int)passes.size()) return false;
         const PassSpec &ps = passes[kv.first];
         if (ps.E != kv.second.first || ps.tile != kv.second.second) return false;  // not applied
-        PassArgs a{};
+        TileArgs a{};
         a.npencils = 0;  // an empty launch returns before running
         if (launch(dtype, ps, nullptr, nullptr, a, 0) == cudaErrorInvalidValue) return false;
     }
@@ -1460,7 +1460,7 @@ int Plan::run(const void *in, void *out, cudaStream_t st) {
                               : p.src == SRC_OUT ? (const char *)out + off
                                                  : (const char *)work;
             char *dst = p.dst == DST_OUT ? (char *)out + off : (char *)work;
-            PassArgs a = pass_args(p, p.npencils_per_batch * nb);
+            TileArgs a = pass_args(p, p.npencils_per_batch * nb);
             a.elems = p.transform_elems * nb;
             prof_begin(st);
             cudaError_t e = launch(dtype, p, src, dst, a, st);
@@ -1471,8 +1471,8 @@ int Plan::run(const void *in, void *out, cudaStream_t st) {
     return WSFFT_SUCCESS;
 }
 
-PassArgs Plan::pass_args(const PassSpec &p, int64_t npencils) const {
-    PassArgs a{};
+TileArgs Plan::pass_args(const PassSpec &p, int64_t npencils) const {
+    TileArgs a{};
     a.npencils = npencils;
     a.inner = p.inner;
     a.log_inner = ilog2(p.inner);
@@ -1573,7 +1573,7 @@ int Plan::run_host_pipelined(const void *hin, void *hout, cudaStream_t st) {
         char *ho = (char *)hout + b * elems * eb;
         char *db = dev + b * elems * eb;
         auto run_pass = [&](const PassSpec &p, char *ptr, int64_t npencils) {
-            const PassArgs a = pass_args(p, npencils);
+            const TileArgs a = pass_args(p, npencils);
             prof_begin(st);
             cudaError_t e = launch(dtype, p, ptr, ptr, a, st);
             prof_end(st);
@@ -1712,7 +1712,7 @@ int Plan::rag_run_grouped(const void *const *in, void *const *out, cudaStream_t 
     auto run_groups = [&](size_t from, size_t to) {
         for (size_t i = from; i < to; ++i) {
             const RagGroup &g = rag_groups[i];
-            PassArgs a{};
+            TileArgs a{};
             a.tiles = g.tiles;
             a.refs = static_cast<const RagRef *>(rag_refs) + g.ref0;
             a.inst = static_cast<const RagInst *>(rag_inst);
@@ -2132,7 +2132,7 @@ int wsfft_plan_set_pass_variant(wsfft_plan plan, int pass, int values_per_thread
     const PassSpec &ps = p->passes[pass];
     if (ps.kind != PASS_CONTIG && ps.kind != PASS_STRIDED) return WSFFT_ERR_UNSUPPORTED;
     // probe: is this shape instantiated?  (an empty launch returns before running)
-    PassArgs a{};
+    TileArgs a{};
     a.npencils = 0;
     PassSpec probe = ps;
     probe.E = values_per_thread;
