@@ -18,14 +18,17 @@ struct OctantRoot {
 };
 // Those met so far: the tables of a plan repeat a few hundred angles thousands
 // of times, at half a microsecond (128-bit long double) each.  Orders up to
-// 4096 share a table of that order's octant; longer ones are looked up by
-// their angle in units of (pi/4) 2^-32.
+// 4096 share a table of that order's octant, and one of its roots in float;
+// longer ones are looked up by their angle in units of (pi/4) 2^-32.
 struct RootMemo {
     static constexpr int LOG_ORDER = 12;
     OctantRoot near[(1 << (LOG_ORDER - 3)) + 1];
     bool known[(1 << (LOG_ORDER - 3)) + 1] = {};
+    float2 circle[1 << LOG_ORDER];
+    bool on_circle[1 << LOG_ORDER] = {};
     std::unordered_map<int64_t, OctantRoot> far;
 };
+
 // exp(-2*pi*i*m/n), n a power of two: the angle is reduced to the first octant by the
 // eight-fold symmetry of the unit circle, evaluated in long double, then
 // rounded to float (twiddles computed in higher precision and rounded once).

@@ -96,10 +96,20 @@ OctantRoot fold(int64_t m, int64_t n, RootMemo *memo, int &octant) {
 }  // namespace
 
 float2 host_root(int64_t m, int64_t n, RootMemo *memo) {
-    int o;
-    const OctantRoot r = fold(m, n, memo, o);
-    const auto cs = unfold(o, r.cf, r.sf);
-    return make_float2(cs.first, cs.second);
+    auto root = [&]() {
+        int o;
+        const OctantRoot r = fold(m, n, memo, o);
+        const auto cs = unfold(o, r.cf, r.sf);
+        return make_float2(cs.first, cs.second);
+    };
+    if (!memo || n > (1 << RootMemo::LOG_ORDER)) return root();
+    const int shift = RootMemo::LOG_ORDER - __builtin_ctzll((unsigned long long)n);
+    const size_t i = ((uint64_t)m << shift) & ((1u << RootMemo::LOG_ORDER) - 1);
+    if (!memo->on_circle[i]) {
+        memo->circle[i] = root();
+        memo->on_circle[i] = true;
+    }
+    return memo->circle[i];
 }
 
 std::complex<double> host_root_d(int64_t m, int64_t n, RootMemo *memo) {
@@ -544,6 +554,7 @@ const float2 *Plan::table2(int N, int R0) {
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
     std::vector<float2> h;
+    h.reserve((size_t)N);
     for (int r = 1; r < N / R0; ++r)
         for (int k = 0; k < R0; ++k) h.push_back(host_root((int64_t)r * k, N, &roots));
     h.push_back(make_float2(0.f, 0.f));
@@ -558,6 +569,7 @@ const float2 *Plan::class_table(int n, int classes) {
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
     std::vector<float2> h;
+    h.reserve((size_t)n);
     for (int y = 1; y < classes; ++y)
         for (int k = 0; k < n / classes; ++k) h.push_back(host_root((int64_t)y * k, n, &roots));
     h.push_back(make_float2(0.f, 0.f));
@@ -572,6 +584,7 @@ const float2 *Plan::wide_table(int zb, int rb) {
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
     std::vector<float2> h;
+    h.reserve((size_t)2 << zb);
     int64_t ns = (int64_t)1 << (5 - rb);
     for (int R : {32, (1 << zb) / (32 << (5 - rb))}) {
         for (int r = 1; r < R; ++r)

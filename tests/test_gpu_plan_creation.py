@@ -1,8 +1,8 @@
 """What a plan costs to create: the tables of the fused, wide and grouped
 schedules add little to those of one launch per axis.  Each pair compares a
-plan that has them with one of the same library that does not, median of nine;
-before the tables shared their roots, their memory and their copy the ratios
-were 2.9, 1.3, 2.5 and 2.0."""
+plan that has them with one of the same library that does not, the least of
+nine (what else runs on the host only adds); before the tables shared their
+roots, their memory and their copy the ratios were 2.9, 1.3, 2.5 and 2.0."""
 import time
 
 import numpy as np
@@ -23,7 +23,7 @@ def _lib():
     torch.zeros(1, device="cuda")
 
 
-def _median(make):
+def _least(make):
     times = []
     for _ in range(9):
         torch.cuda.synchronize()
@@ -31,13 +31,13 @@ def _median(make):
         plan = make()
         times.append(time.perf_counter() - t)
         plan.close()
-    return sorted(times)[4]
+    return min(times)
 
 
 @pytest.mark.parametrize("dims,plain", [((4096, 4096), (4096, 256)), ((128, 128, 128), (256, 256, 256))])
 def test_split_axes(dims, plain):
     W.Plan(plain).close()
-    assert _median(lambda: W.Plan(dims)) < 1.15 * _median(lambda: W.Plan(plain))
+    assert _least(lambda: W.Plan(dims)) < 1.15 * _least(lambda: W.Plan(plain))
 
 
 @pytest.mark.parametrize("count", [64, 256])
@@ -46,4 +46,4 @@ def test_ragged_groups(count):
     shapes = [tuple(int(v) for v in s) for s in rng.choice(np.asarray((32, 64, 128, 256)), size=(count, 3))]
     W.RaggedPlan(shapes, W.C32).close()
     # 16-bit storage: the queue alone
-    assert _median(lambda: W.RaggedPlan(shapes, W.C32)) < 1.75 * _median(lambda: W.RaggedPlan(shapes, W.C16F))
+    assert _least(lambda: W.RaggedPlan(shapes, W.C32)) < 1.75 * _least(lambda: W.RaggedPlan(shapes, W.C16F))
