@@ -343,14 +343,27 @@ def run_reference(args, world, rank):
     print(json.dumps(line), flush=True)
 
 
+def launches_of(plan, execute) -> int:
+    """Kernel launches that one call of `execute` makes on `plan`, from the
+    plan's own recording: the schedule depends on the storage type, the batch
+    and whether the call is in place, which Plan.passes() does not know."""
+    torch.cuda.synchronize()
+    plan.profile(256)
+    execute()
+    n = len(plan.launch_times(256))
+    plan.profile(0)
+    return n
+
+
 def sizes_leg(W, dev, stream, hbm_peak, steps=20, warmup=3):
     """The other transform sizes of the workload family, each timed like the
     main step ((FFT + IFFT)/2 per execute of the whole batch, data resident,
     CUDA events on the stream): cubes 32^3 (the small configuration:
-    latency-bound, three launches), 128^3, 256^3 and 1024^3 (complex64 and
+    latency-bound), 128^3, 256^3 and 1024^3 (complex64 and
     float16 storage), 2D
-    4096 x 4096 and 1D 2^20 x batch 512 (complex64).  GB/s counts one read and
-    one write of the array per launch; the minimum-bytes fraction uses 2
+    4096 x 4096 and 1D 2^20 x batch 512 (complex64).  The forward runs out of
+    place and the inverse in place, whose schedules differ; GB/s counts one
+    read and one write of the array for each launch that they made; the minimum-bytes fraction uses 2
     passes for 2D and 3D and 1 for 1D.  Arrays of 16 MiB (128^3) sit in L2:
     no roofline claim there; those sizes are also timed replayed from a
     captured CUDA graph."""
@@ -370,14 +383,16 @@ def sizes_leg(W, dev, stream, hbm_peak, steps=20, warmup=3):
         norm = W.NORM_PAPER if code == W.C32 else W.NORM_ORTHO
         f = W.Plan(dims, code, W.FORWARD, batch, norm)
         i = W.Plan(dims, code, W.INVERSE, batch, norm)
-        npass = f.passes()[0]
         ms = timed_pairs(f, i, xs, ys, steps, warmup, 1, stream)
+        nf = launches_of(f, lambda: f.execute(xs.data_ptr(), ys.data_ptr(), stream))
+        ni = launches_of(i, lambda: i.execute(ys.data_ptr(), ys.data_ptr(), stream))
         us = ms / steps * 1e3 / 2
         nbytes = elems * eb
         min_passes = 1 if len(dims) == 1 else 2
         rec = {"dims": list(dims), "batch": batch, "dtype": "complex64" if code == W.C32 else "float16 storage",
-               "us_per_execute": round(us, 2), "us_per_transform": round(us / batch, 3), "passes_used": npass,
-               "gb_per_s": round(npass * 2 * nbytes / (us * 1e-6) / 1e9, 1),
+               "us_per_execute": round(us, 2), "us_per_transform": round(us / batch, 3),
+               "launches_forward": nf, "launches_inverse_in_place": ni,
+               "gb_per_s": round((nf + ni) * nbytes / (us * 1e-6) / 1e9, 1),
                "gflops": round(5 * elems * np.log2(elems / batch) / (us * 1e-6) / 1e9, 1)}
         if nbytes > 256 * 2 ** 20:
             rec["min_bytes_roofline_frac"] = round(min_passes * 2 * nbytes / (hbm_peak * 1e9) / (us * 1e-6), 4)
@@ -458,12 +473,15 @@ def autograd_leg(W, dev, stream, steps=20, warmup=3):
     e1.record(stream)
     torch.cuda.synchronize()
     t_pair = e0.elapsed_time(e1) / steps * 1e3
+    trips = launches_of(fwd, lambda: fwd.execute(xd.data_ptr(), y.data_ptr(), stream))
+    trips += launches_of(adj, lambda: adj.execute(y.data_ptr(), y.data_ptr(), stream))
     fwd.close()
     adj.close()
     nbytes = 8 * 128 ** 3 * 8
     return {"shape": list(shape), "dtype": "complex64", "us_per_step_fwd_bwd": round(t_step, 2),
             "us_forward_plus_adjoint_transforms": round(t_pair, 2),
-            "transforms_gb_per_s_3pass": round(2 * 3 * 2 * nbytes / (t_pair * 1e-6) / 1e9, 1),
+            "transforms_launches": trips,
+            "transforms_gb_per_s": round(trips * 2 * nbytes / (t_pair * 1e-6) / 1e9, 1),
             "note": "step includes torch's elementwise loss and its gradient; the 128 MiB batch sits in L2"}
 
 
@@ -493,7 +511,10 @@ def ragged_leg(W, dev, stream, reps=5):
     """The ragged configuration (256 uneven 3D shapes from seed 4, N(0,1)):
     the plan's launches replayed from a captured CUDA graph, as created and
     after wsfft_autotune, vs one plan execute per instance.  launches_batch
-    counts a large instance's plan as one."""
+    counts a large instance's plan as one.  hbm_gbs counts one read and one
+    write of an instance for each trip that the tuned schedule makes over it:
+    three on the queue, otherwise two, or those of a plan of its own from
+    2^17 elements up (smaller ones make three there)."""
     from paper_2209_15040_gb300 import inputs
     shapes = inputs.ragged_shapes(256, 4)
     g = torch.Generator(device=dev)
@@ -503,7 +524,8 @@ def ragged_leg(W, dev, stream, reps=5):
         xs.append(torch.view_as_complex(torch.randn(tuple(int(v) for v in s) + (2,), generator=g,
                                                     device=dev)).contiguous())
         ys.append(torch.empty_like(xs[-1]))
-    elems = int(sum(int(np.prod(s)) for s in shapes))
+    sizes = [int(np.prod(s)) for s in shapes]
+    elems = sum(sizes)
     ins, outs = [x.data_ptr() for x in xs], [y.data_ptr() for y in ys]
     plan = W.RaggedPlan(shapes, W.C32, W.FORWARD)
     # the default (grouped launches), then the autotuned choice (grouped, or
@@ -532,7 +554,10 @@ def ragged_leg(W, dev, stream, reps=5):
     lib.wsfft_plan_launch_times(plan.handle, None, 0, ctypes.byref(count))
     lib.wsfft_plan_profile(plan.handle, 0)
     plans = [W.Plan(tuple(int(v) for v in s), W.C32, W.FORWARD, 1) for s in shapes]
-    launches = sum(p.passes()[0] for p in plans)
+    launches = [launches_of(p, lambda: p.execute(i, o, stream)) for p, i, o in zip(plans, ins, outs)]
+    trips = [3 if not tune.get("grouped") else 2 if n < 1 << 17 else k for k, n in zip(launches, sizes)]
+    moved = sum(t * 2 * n * 8 for t, n in zip(trips, sizes))
+
     def per_instance():
         for p, i, o in zip(plans, ins, outs):
             p.execute(i, o, stream)
@@ -550,11 +575,11 @@ def ragged_leg(W, dev, stream, reps=5):
         p.close()
     plan.close()
     return {"instances": len(shapes), "elements": elems, "bytes": elems * 8,
-            "persistent_graph_us": round(t_graph, 1), "persistent_graph_default_us": round(t_default, 1),
+            "graph_us": round(t_graph, 1), "graph_default_us": round(t_default, 1),
             "autotuned": tune, "per_instance_us": round(t_inst, 1),
             "speedup": round(t_inst / t_graph, 3), "launches_batch": count.value,
-            "launches_per_instance": launches,
-            "hbm_gbs_3pass_equiv": round(3 * 2 * elems * 8 / (t_graph * 1e-6) / 1e9, 1)}
+            "launches_one_plan_per_instance": sum(launches),
+            "hbm_gbs": round(moved / (t_graph * 1e-6) / 1e9, 1)}
 
 
 def run_sweep(args):
