@@ -230,7 +230,8 @@ int wsfft_destroy(wsfft_plan plan);
  * (bounded) until the previous superstep of the same instance is complete.
  * WSFFT_C32 executes out of place run grouped launches instead: one per tile
  * shape and trip over all instances that have it, two trips per instance
- * (instances of more than 2^22 elements: three, one after the other).
+ * (instances of more than 2^22 elements and 32 x 256 x 64: three, one after the
+ * other).
  * Section 4.4 (more than one pencil per processor) generalised to one thread
  * block per tile.  Normalisation as wsfft_plan_create (PAPER for WSFFT_C32,
  * ORTHO otherwise).  The launches and their table upload can be captured in a
@@ -285,9 +286,10 @@ int wsfft_plan_set_ragged_variant(wsfft_plan plan, int shape_select, int lag);
  * butterflies run as packed FP32x2 instructions; tile code 2000 selects the
  * tensor-core contiguous superstep (16-bit storage, N = 512; the
  * values-per-thread argument is then ignored); tile codes 4013 and 4014
- * select the pipelined strided kernel with 2^13 or 2^14 elements per tile
- * (values per thread: the radix of its first stage, 8 up to 64 points, 16 up
- * to 256, 32 above).  Used by the autotuner.
+ * select the pipelined kernels with 2^13 or 2^14 elements per tile: strided and
+ * transposing supersteps, and (4013) contiguous ones of 32..256 points (values
+ * per thread: the radix of their first stage, 8 up to 64 points, 16 for 128,
+ * 256, 2048 and 4096, 32 for 512 and 1024).  Used by the autotuner.
  * Errors: INVALID_ARG, UNSUPPORTED (that shape is not built for this pass).
  * A shape that needs whole tiles (either pencil-pair kernel, the pipelined
  * kernel) on a pass whose pencil count or stride is not a multiple of its
@@ -296,14 +298,21 @@ int wsfft_plan_set_pass_variant(wsfft_plan plan, int pass, int values_per_thread
 
 /* Choose the schedule of a rank-3 transform n0 x n x n (n in {128, 256, 512,
  * 1024}, any n0; the pipelined engine needs n0 == n):
- *   0 (default): one launch per superstep (three trips through HBM); for
- *      rank-2 and rank-3 transforms with a last axis of 32..256 points whose
- *      inner two axes hold at most 2^13 elements those two take one launch and
- *      one trip, and rank-3 transforms of up to 2^22 elements take two trips
- *      out of place where their axes allow; a strided axis of 2048 or 4096
- *      points (or 1024 far apart) gives its first digit to the last axis'
- *      launch, out of place (in place, from host buffers and with a chosen
- *      pass shape: one launch per superstep; the results agree up to rounding);
+ *   0 (default): one launch per superstep (three trips through HBM), except
+ *      a. rank-2 and rank-3 transforms with a last axis of 32..256 points whose
+ *         inner two axes hold at most 2^13 elements: those two take one launch
+ *         and one trip (the whole call from 2^17 elements up, WSFFT_C32 slabs of
+ *         32 x 32 from 2^15), in place, out of place and, where
+ *         wsfft_execute_host does not overlap its copies, from host buffers;
+ *      b. rank-3 transforms of up to 2^22 elements with larger slabs whose axes
+ *         allow it: two trips, out of place (the whole call from 2^17 elements up);
+ *      c. a strided axis of 2048 or 4096 points (or 1024 far apart), from 2^20
+ *         elements up (2^21 in 16-bit storage): its first digit goes with the
+ *         last axis' launch, out of place.
+ *      With a chosen pass shape, and for b and c in place or from host buffers:
+ *      one launch per superstep.  Which kernels run depends on the number of
+ *      elements of the whole call, so a transform alone, the same one in a batch,
+ *      in place and out of place agree up to rounding, not bit for bit;
  *   4 (n in {256, 512}): two trips through HBM -- one thread-block cluster
  *      per n x n slab runs its z superstep, meets at a cluster barrier, and
  *      runs its y superstep on the slab as the z tiles left it in L2; then
@@ -339,10 +348,11 @@ int wsfft_plan_sync_status(wsfft_plan plan, wsfft_stream stream);
 
 /* Number of passes over the array of the plan's schedule (one per superstep,
  * or the schedule chosen by wsfft_plan_set_engine), and the minimum number of
- * bytes one execute reads plus writes in HBM for it.  Device executes of
- * rank-2 and rank-3 transforms whose inner axes fit on a processor's tile make
- * one pass less (wsfft_plan_set_engine, mode 0); wsfft_plan_launch_times lists
- * the launches an execute made. */
+ * bytes one execute reads plus writes in HBM for it.  This is the schedule
+ * whose passes wsfft_plan_set_pass_variant counts; under mode 0 of
+ * wsfft_plan_set_engine an execute of form a or b makes one pass less, one of
+ * form c as many.  wsfft_plan_launch_times lists the launches that an execute
+ * made. */
 int wsfft_plan_passes(wsfft_plan plan, int *passes, int64_t *bytes_per_execute);
 
 /* Per-launch timing (the paper times compute and communication phases

@@ -366,8 +366,9 @@ int pipe_tile_bits_variant(int dtype, int64_t N, int64_t rows, int64_t total, bo
 // Whether a rank-2 or rank-3 transform (axes d) runs its inner axes fused on
 // the tile kernels (tile_fused.cuh).  A fused trip replaces two (the inner
 // axes of slabs of up to 2^13 elements) or turns three trips into two, and wins
-// at every size measured, from one small transform (a launch less) to 1 GiB
-// (2^27 elements, complex64 / FP16 storage, us):
+// from 2^17 elements up (below, see build_fused: a tile keeps one block busy for
+// longer than separate launches take) to 1 GiB (2^27 elements, complex64 / FP16
+// storage, us):
 //   64 x 64 batches 329 / 262 against 597 / 464, 32^3 623 / 410 against 962 /
 //   771, 64^3 631 / 431 against 896 / 708; split middle axis: 128^3 684 / 458
 //   against 919 / 734 (one cube 15.3 against 18.9), 64 x 256^2 687 / 474
