@@ -350,6 +350,17 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         if (tile < ntiles) rag_next = rag_tile(a, tile);
     if (tile < ntiles) issue(tile);
     cp_async_commit();
+    // Where every block has one tile and an SM to itself, the next launch may come in
+    // now and not only with the last stage: its ramp (about 1.5 us) was a fifth of a
+    // small call.  Back to back, us, with one launch per axis in brackets: complex64
+    // 64^3 8.7 -> 7.6 (8.0), eight of 8 x 128 x 64 9.6 -> 7.8 (7.3), 64 x 128 x 128 11.7 -> 10.8
+    // (15.1); 16-bit storage 64^3 8.5 -> 7.1 (7.7), 64 x 256 x 32 10.4 -> 7.4 (8.0).  With more
+    // tiles the next launch's blocks get in the way: 256 tiles of 128^3 in 16-bit
+    // storage 12.9 -> 14.9; complex64 before the general strided kernel 128 tiles of 128 x
+    // 128 x 64 11.0 -> 13.1, 80 of 32 x 64 x 64 8.9 -> 10.1, and 16 take 3-6% longer.
+    if constexpr (!RAG)
+        if (sizeof(S) == 4 || a.log_y0 > 0 ? ntiles <= 128 : ntiles >= 32 && ntiles <= 64)
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (; tile < ntiles; tile += gridDim.x) {
         cpair v[32];
         if constexpr (RAG) {
@@ -452,6 +463,9 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
         if (tile < ntiles) rag_next = rag_tile(a, tile);
     if (tile < ntiles) issue(tile);
     cp_async_commit();
+    // as in tile_slab_kernel
+    if constexpr (!RAG)
+        if (ntiles <= 128) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (; tile < ntiles; tile += gridDim.x) {
         cpair v[32];
         if constexpr (RAG) {
