@@ -28,8 +28,8 @@ cudaError_t launch_tile_c16bf(int mode, int N, int tb, const void *in, void *out
 
 // Fused tile kernels (tile_fused.cuh), tiles of 2^13 elements.
 constexpr int FUSED_TILE_BITS = 13;
-// Below this many elements 32 x 32 slabs run in tiles of 2^11 (complex64), others
-// one launch per axis.
+// Up to this many elements 32 x 32 slabs run in tiles of 2^11 (complex64), others
+// one launch per axis (Plan::build_fused).
 constexpr int64_t FUSED_SMALL_ELEMS = (int64_t)1 << 17;
 constexpr int FUSED_SMALL_BITS = 11;
 

@@ -37,7 +37,7 @@ cudaError_t WSFFT_SLAB_TILE_NAME(int zb, int yb, const void *in, void *out, cons
     // time of one block of four.  32^3: 5.21 us captured and 5.65 in a loop of
     // calls against 6.21 and 6.61 with tiles of 2^13.
     if constexpr (sizeof(S) == 8)
-        if (a.elems < FUSED_SMALL_ELEMS && zb == 5 && yb == 5) {
+        if (a.elems <= FUSED_SMALL_ELEMS && zb == 5 && yb == 5) {
             using G = TileSlab<FUSED_SMALL_BITS, 5, 5>;
             a.tiles = (a.elems + (1 << FUSED_SMALL_BITS) - 1) >> FUSED_SMALL_BITS;
             return launch_fused<G>(tile_slab_kernel<G, S, true>, in, out, a, st);

@@ -295,13 +295,20 @@ bool override_usable(int E, int tile, int N) {
 // kernels; 0: the one-tile-per-block kernels are faster, or the pencils do
 // not fill whole tiles.  Measured per superstep, against those kernels:
 //   2048 points, three stages, 64-byte rows (complex64): 508-587 us against
-//     566-603, 16-bit 383-431 against 466-481; 4096 points only in 16-bit storage
-//     (583-662 against 631-704; complex64 732 against 696).
+//     566-603, 16-bit 383-431 against 466-481.
+//   4096 points: only in 16-bit storage, from 2^25 elements up and at strides of
+//     32 to 1024 elements (in place 582-592 us against 595-611, out of place 600-627
+//     against 608-639; 2^25 152-155 against 153-156).  Smaller arrays, and strides
+//     of 4 to 16 elements, whose general kernels read whole runs, were slower
+//     on the tiles (2^23 at a stride of 8: 40.8 us against 33.0, of 256: 42.4 against
+//     40.4; 2^26 at 8: 267 against 237), wide strides no faster (2^26 at 2^14: 337 against
+//     330); complex64 732 against 696.
 //   complex64, 1024 points (shorter axes are at the copy rate without them):
 //     tiles of 2^13 elements up to a stride of 2^16 elements from 2^22
 //     elements up (2^22 12.4 us against 14.4, 2^24 48-50 against 53-57, 2^25
-//     89-92 against 99-108); for large arrays or wider strides their 64-byte
-//     rows cost too much (2^27: 349-372 us, and 540 at a stride of 2^17) and
+//     89-92 against 99-108; at a stride of 8, where the general kernel reads whole
+//     runs, 2^22 11.1 against 12.4 but 2^25 93.7 against 82.9); for large arrays or
+//     wider strides their 64-byte rows cost too much (2^27: 349-372 us, and 540 at a stride of 2^17) and
 //     tiles of 2^14 (128-byte rows) take over (2^27 351-388 us against 373-467).
 //   16-bit storage: from 2^22 elements up (2^27 170-174 us against 224-273
 //     at 32..128 points, 185-206 against 235-251 at 256, 200-212 against
@@ -313,10 +320,11 @@ bool override_usable(int E, int tile, int N) {
 int pipe_tile_bits(int dtype, int64_t N, int64_t inner, int64_t total) {
     int tb = 0;
     if (N == 2048) tb = total >= ((int64_t)1 << 22) ? 14 : 0;
-    if (N == 4096 && dtype != WSFFT_C32) tb = total >= ((int64_t)1 << 23) ? 14 : 0;
+    if (N == 4096 && dtype != WSFFT_C32)
+        tb = total >= ((int64_t)1 << 25) && inner >= 32 && inner <= 1024 ? 14 : 0;
     if (dtype == WSFFT_C32) {
         if (N == 1024 && inner <= ((int64_t)1 << 16) && total < ((int64_t)1 << 27))
-            tb = total >= ((int64_t)1 << 22) ? 13 : 0;
+            tb = total >= ((int64_t)1 << 22) && (inner >= 16 || total < ((int64_t)1 << 25)) ? 13 : 0;
         else if (N == 1024 && total >= ((int64_t)1 << 25))
             tb = 14;
     } else if (total >= ((int64_t)1 << 22)) {

@@ -1,0 +1,53 @@
+"""Calls next to the limits of the tile kernels' rules, where the general kernels are the
+faster ones: the schedule they run, told by launches or by the bytes of the
+result (the two kernels round differently), and their error."""
+import pytest
+import torch
+
+from paper_2209_15040_gb300 import wsfft as W
+from tests._helpers import DT, TOL
+
+pytestmark = pytest.mark.gpu
+
+
+def _input(shape, dtype):
+    x = torch.randn(*shape, 2, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    return torch.view_as_complex(x) if dtype == "c32" else x.to(torch.float16 if dtype == "c16f" else torch.bfloat16)
+
+
+def _run(plan, x):
+    out = torch.empty_like(x)
+    plan.execute(x.data_ptr(), out.data_ptr())
+    torch.cuda.synchronize()
+    return out
+
+
+def _same(a, b):
+    a, b = (torch.view_as_real(t) if t.is_complex() else t for t in (a, b))
+    return torch.equal(a, b)
+
+
+def _diff(a, b):
+    a, b = (torch.view_as_real(t) if t.is_complex() else t.float() for t in (a, b))
+    return float((a - b).norm() / b.norm())
+
+
+# points, stride, elements, general shape, tiled?
+AXES = [("c16f", 4096, 8, 1 << 23, (16, 0), False), ("c16bf", 4096, 256, 1 << 23, (16, 0), False),
+        ("c16f", 4096, 16, 1 << 25, (16, 0), False), ("c16f", 4096, 4096, 1 << 25, (16, 0), False),
+        ("c16f", 4096, 32, 1 << 25, (16, 0), True), ("c16bf", 4096, 1024, 1 << 25, (16, 0), True),
+        ("c32", 1024, 8, 1 << 25, (16, 3008), False), ("c32", 1024, 8, 1 << 22, (16, 3008), True),
+        ("c32", 1024, 16, 1 << 25, (16, 3008), True)]
+
+
+@pytest.mark.parametrize("dtype, n, inner, elems, general, tiled", AXES)
+def test_strided_axis(dtype, n, inner, elems, general, tiled):
+    batch = elems // (n * inner)
+    x = _input((elems,), dtype)
+    plan = W.AxisPlan(n, inner, DT[dtype], W.FORWARD, batch, W.NORM_ORTHO)
+    default = _run(plan, x)
+    plan.set_pass_variant(0, *general)
+    chosen = _run(plan, x)
+    plan.close()
+    assert _same(default, chosen) != tiled
+    assert _diff(default, chosen) < TOL[dtype]
