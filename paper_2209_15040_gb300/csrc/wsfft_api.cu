@@ -420,8 +420,10 @@ FusedShape fused_tile_rule(const std::vector<int64_t> &d) {
 // 2048^2 684 / 495 against 889 / 741, 64 x 2048 x 1024 677 / 470 against 870 /
 // 827, 1024^3 8100 / 5982 against 8766 / 7126, 1024 x 512^2 1997 against 2107;
 // 1024 x 128 x 1024, whose outer stride is 2^17, 996 / 701 against 986 / 649.
-// Below 2^20 elements (2^21 in 16-bit storage) the three-stage tile's latency
-// costs more (one FP16 2048 x 512: 14.3 against 13.2).
+// Below 2^20 elements (2^21 in 16-bit storage, and 2^21 itself for 2048 points
+// beside 512) the three-stage tile's latency costs more (FP16 2048 x 512: one 14.3
+// against 13.2, two 15.2 against 13.6, three 17.0 against 21.7; 4096 x 512 15.6 against
+// 16.4, 2048 x 1024 15.2 against 16.8).
 struct WideShape {
     int axis = -1, rb = 0;
 };
@@ -434,6 +436,7 @@ WideShape wide_tile_rule(int dtype, const std::vector<int64_t> &d, int64_t total
     // the longest of the axes that qualify; the outer one where both are as long
     for (int ax = r - 2; ax >= 0; --ax) {
         const bool far = r == 3 && ax == 0 && d[0] == 1024 && d[1] * d[2] >= ((int64_t)1 << 18);
+        if (dtype != WSFFT_C32 && zb == 9 && d[ax] == 2048 && total <= ((int64_t)1 << 21)) continue;
         if ((d[ax] >= 2048 || far) && (w.axis < 0 || d[ax] >= d[w.axis])) w.axis = ax;
     }
     if (w.axis < 0) return w;

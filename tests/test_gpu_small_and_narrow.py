@@ -51,3 +51,16 @@ def test_strided_axis(dtype, n, inner, elems, general, tiled):
     plan.close()
     assert _same(default, chosen) != tiled
     assert _diff(default, chosen) < TOL[dtype]
+
+
+@pytest.mark.parametrize("dims, batch, wide", [((2048, 512), 2, False), ((2048, 512), 3, True),
+                                               ((4096, 512), 1, True), ((2048, 1024), 1, True)])
+def test_digit_of_2048_points_beside_512(dims, batch, wide):
+    x = _input((batch,) + dims, "c16f")
+    plan = W.Plan(dims, W.C16F, W.FORWARD, batch)
+    default = _run(plan, x)
+    plan.set_engine(4)  # one launch per superstep for this shape
+    chosen = _run(plan, x)
+    plan.close()
+    assert _same(default, chosen) != wide
+    assert _diff(default, chosen) < TOL["c16f"]
