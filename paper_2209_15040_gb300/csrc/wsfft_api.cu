@@ -665,13 +665,17 @@ int Plan::build_fused(const std::vector<int64_t> &d, bool inv) {
     if (!f.use) return WSFFT_SUCCESS;
     // Below 2^17 elements a block's time for 2^13 elements (about 4 us) is more than
     // two launches over many small blocks take: one 64 x 64 plane 5.5 us against
-    // 3.1, 32 x 32 x 64 6.3 against 5.1 (2^17 and more: 64^3 7.1 against 9.1, eight
-    // 32^3 6.7 against 11.1).  The smaller tiles of 32 x 32 slabs make up for that
-    // from 2^15 elements up in complex64: 32^3 5.2 us either way, one launch fewer.
-    const int64_t total = elems * batch;
-    if (total < FUSED_SMALL_ELEMS && !(dtype == WSFFT_C32 && f.zb + f.yb == 10 && total >= FUSED_SMALL_ELEMS / 4))
-        return WSFFT_SUCCESS;
+    // 3.1, 32 x 32 x 64 6.3 against 5.1.  At 2^17 itself the same holds in complex64
+    // and for rank 3 (back to back and captured: 32 x 64 x 64 7.1 and 7.2 against 5.7 and
+    // 5.1, thirty-two 64 x 64 planes 5.1 and 5.4 against 4.0 and 3.6; in 16-bit storage slabs
+    // of 2^13 elements take 4.3 us either way).  Above: 64^3 7.6 against 8.0, eight 32^3
+    // 7.0 against 9.6; up to 2^18 elements a launch less for the host, at up to 1.2 us more
+    // on the GPU (twenty-four 128 x 64 planes 5.3 against 4.4).  The smaller tiles of 32 x 32 slabs make up for it from 2^15 to 2^17
+    // elements in complex64: 32 planes 3.7 against 4.0, 32^3 5.5 against 5.8.
     const int r = (int)d.size();
+    const int64_t total = elems * batch;
+    const bool small = total < FUSED_SMALL_ELEMS || (total == FUSED_SMALL_ELEMS && (dtype == WSFFT_C32 || r == 3));
+    if (small && !(dtype == WSFFT_C32 && f.zb + f.yb == 10 && total >= FUSED_SMALL_ELEMS / 4)) return WSFFT_SUCCESS;
     const int64_t n1 = d[r - 2], n2 = d[r - 1], n0 = r == 3 ? d[0] : 1;
     const int64_t rows = (int64_t)1 << f.yb;
     PassSpec a{};

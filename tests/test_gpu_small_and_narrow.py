@@ -64,3 +64,21 @@ def test_digit_of_2048_points_beside_512(dims, batch, wide):
     plan.close()
     assert _same(default, chosen) != wide
     assert _diff(default, chosen) < TOL["c16f"]
+
+
+# 2^17 elements and next to them: one launch per axis where that is the faster
+@pytest.mark.parametrize("dtype, dims, batch, launches", [
+    ("c32", (32, 64, 64), 1, 3), ("c32", (64, 64), 32, 2), ("c32", (64, 64), 33, 1), ("c32", (2, 64, 128), 8, 3),
+    ("c32", (32, 32), 128, 1), ("c32", (32, 32, 32), 4, 2), ("c32", (32, 32), 127, 1),
+    ("c16f", (32, 64, 64), 1, 3), ("c16bf", (8, 128, 64), 2, 3), ("c16f", (64, 64), 32, 1)])
+def test_fused_from_2_17_elements(dtype, dims, batch, launches):
+    x = _input((batch,) + dims, dtype)
+    for direction in (W.FORWARD, W.INVERSE):
+        plan = W.Plan(dims, DT[dtype], direction, batch, W.NORM_ORTHO)
+        plan.profile(8)
+        default = _run(plan, x)
+        assert len(plan.launch_times()) == launches
+        plan.profile(0)
+        plan.set_engine(4)
+        assert _diff(default, _run(plan, x)) < TOL[dtype]
+        plan.close()
