@@ -1007,8 +1007,14 @@ int Plan::make_schedule() {
             p.tile = PIPE_TILE + FUSED_TILE_BITS;
         }
         if (p.kind == PASS_STRIDED) {
-            // pipelined tile kernels (tile.cuh) where whole tiles fit
-            const int tb = pipe_tile_bits(dtype, p.N, inner, elems * batch);
+            // pipelined tile kernels (tile.cuh) where whole tiles fit; in 16-bit storage
+            // not right after a contiguous superstep of 2048 or 4096 points while a few
+            // tiles are a second wave (512 x 2048 FP16: 2^22 elements, 512 tiles for 456
+            // resident blocks, 22.9 us against 20.4; 128 x 2048 in a batch of 20 23.6 against
+            // 22.6; 1.5 * 2^22 elements 27.2 against 29.1; 1024 points are faster at each size)
+            const bool held = dtype != WSFFT_C32 && axis_inner == 0 && p.N <= 512 && r >= 2 && inner == d[r - 1] &&
+                              inner >= 2048 && elems * batch <= ((int64_t)5 << 20);
+            const int tb = held ? 0 : pipe_tile_bits(dtype, p.N, inner, elems * batch);
             if (tb) {
                 p.E = tile_table_E(p.N);
                 p.tile = PIPE_TILE + tb;

@@ -53,6 +53,23 @@ def test_strided_axis(dtype, n, inner, elems, general, tiled):
     assert _diff(default, chosen) < TOL[dtype]
 
 
+# a strided superstep right after rows of 2048 or 4096 points, 16-bit storage
+@pytest.mark.parametrize("dims, batch, general, tiled", [((512, 2048), 4, (16, 3016), False),
+                                                         ((512, 4096), 2, (16, 3016), False),
+                                                         ((128, 2048), 20, (16, 0), False),
+                                                         ((512, 2048), 6, (16, 3016), True),
+                                                         ((512, 1024), 8, (16, 3016), True)])
+def test_after_long_rows(dims, batch, general, tiled):
+    x = _input((batch,) + dims, "c16f")
+    plan = W.Plan(dims, W.C16F, W.FORWARD, batch)
+    default = _run(plan, x)
+    plan.set_pass_variant(1, *general)
+    chosen = _run(plan, x)
+    plan.close()
+    assert _same(default, chosen) != tiled
+    assert _diff(default, chosen) < TOL["c16f"]
+
+
 @pytest.mark.parametrize("dims, batch, wide", [((2048, 512), 2, False), ((2048, 512), 3, True),
                                                ((4096, 512), 1, True), ((2048, 1024), 1, True)])
 def test_digit_of_2048_points_beside_512(dims, batch, wide):
