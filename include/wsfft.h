@@ -301,13 +301,13 @@ int wsfft_plan_set_pass_variant(wsfft_plan plan, int pass, int values_per_thread
  *   0 (default): one launch per superstep (three trips through HBM), except
  *      a. rank-2 and rank-3 transforms with a last axis of 32..256 points whose
  *         inner two axes hold at most 2^13 elements: those two take one launch
- *         and one trip (the whole call from 2^17 elements up, WSFFT_C32 slabs of
- *         32 x 32 from 2^15), in place, out of place and, where
+ *         and one trip (the whole call above 2^17 elements; 16-bit planes from
+ *         2^17, WSFFT_C32 slabs of 32 x 32 from 2^15), in place, out of place and, where
  *         wsfft_execute_host does not overlap its copies, from host buffers;
  *      b. rank-3 transforms of up to 2^22 elements with larger slabs whose axes
- *         allow it: two trips, out of place (the whole call from 2^17 elements up);
+ *         allow it: two trips, out of place (the whole call above 2^17 elements);
  *      c. a strided axis of 2048 or 4096 points (or 1024 far apart), from 2^20
- *         elements up (2^21 in 16-bit storage): its first digit goes with the
+ *         elements up (in 16-bit storage 2^21, and more for 2048 beside 512): its first digit goes with the
  *         last axis' launch, out of place.
  *      With a chosen pass shape, and for b and c in place or from host buffers:
  *      one launch per superstep.  Which kernels run depends on the number of

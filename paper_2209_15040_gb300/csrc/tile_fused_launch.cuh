@@ -34,8 +34,8 @@ cudaError_t WSFFT_SLAB_TILE_NAME(int zb, int yb, const void *in, void *out, cons
     TileArgs a = arg;
     // Few tiles (complex64 slabs of 2^10): a quarter of a tile's elements per
     // block, one warp each; loads, exchanges and stores take a quarter of the
-    // time of one block of four.  32^3: 5.21 us captured and 5.65 in a loop of
-    // calls against 6.21 and 6.61 with tiles of 2^13.
+    // time of one block of four.  Four 32^3: 5.7 us back to back and 5.6 captured
+    // against 6.6 and 6.7 with tiles of 2^13.
     if constexpr (sizeof(S) == 8)
         if (a.elems <= FUSED_SMALL_ELEMS && zb == 5 && yb == 5) {
             using G = TileSlab<FUSED_SMALL_BITS, 5, 5>;
