@@ -334,8 +334,8 @@ struct TileSmem {
     static constexpr int LOAD = G::LBUF * (int)sizeof(S), XCHG = tile_xfloats<G>() * (FULL ? 8 : 4);
     static constexpr int X = SHARED_BUF ? 0 : LOAD;
     static constexpr int TW = SHARED_BUF ? (LOAD > XCHG ? LOAD : XCHG) : LOAD + XCHG;
-    // 16-bit storage is bound by the SM and reads its stage twiddles 5%
-    // faster from shared memory; complex64 is bound by HBM and was slower so
+    // 16-bit storage reads its stage twiddles 5% faster from shared memory;
+    // complex64 was slower so
     static constexpr bool SHARED_TW = sizeof(S) == 4;
     static constexpr int C = TW + (SHARED_TW ? G::TABLE * 8 : 0);
     static constexpr int TILE_C = TWID ? G::W * (8 << G::R0) : 0, TILE_U = TWID ? G::W * (8 << G::R1) : 0;
@@ -350,9 +350,10 @@ struct TileSmem {
 //     long); 0.343 ms against 0.410 (8 pencils, 64-byte rows) and 0.49-0.51
 //     (16 pencils, one block per SM without the copies in flight) at a stride
 //     of 2^10, 0.39 against 0.46-0.50 at 2^17;
-//   16-bit storage: the SM -- FP32 pipe and shared memory, which the blocks
-//     of an SM overlap in part: 512 points 0.20 ms (tiles of 2^13), 0.227
-//     (2^14) against 0.26-0.27; 256 points 0.187 and 0.205 against 0.24-0.25.
+//   16-bit storage: latencies of the FP32 pipe, shared memory and the copies (each
+//     unit 45-56% busy), which the blocks of an SM overlap in part: 512 points
+//     0.20 ms (tiles of 2^13), 0.227 (2^14) against 0.26-0.27; 256 points 0.187 and
+//     0.205 against 0.24-0.25.
 // With the four-step's inter-step twiddle w_L^(q k) on the store (pencil q,
 // k = k1 + Ns r): the product of w_L^(q k1) and w_(L/Ns)^(q r), whose tables
 // hold every q for the few values of k1 and of r, so a tile copies its own

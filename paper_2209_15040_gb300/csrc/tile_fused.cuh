@@ -268,9 +268,11 @@ __device__ __forceinline__ void tile_store(S *p, cpair z, float sx, float sy) {
     SplitPair<S>::store(reinterpret_cast<typename SplitPair<S>::T *>(p), z);
 }
 
-// What bounds it: complex64 the memory system (2^27 elements, read and write:
-// 0.330-0.345 ms, 0.92-0.96 of the copy rate; the two supersteps it replaces
-// 0.60-0.67), 16-bit storage the SM (0.235-0.27 ms against 0.36-0.56).  Two
+// 2^27 elements, read and write: complex64 0.330-0.345 ms, 0.92-0.96 of the copy
+// rate (the two supersteps it replaces 0.60-0.67); 16-bit storage 0.235-0.27 ms
+// (0.36-0.56).  What bounds it: latencies that 8 warps per SM (12 in 16-bit storage)
+// cover in part; in complex64 memory is the busiest unit (67% of the DRAM peak
+// from cold caches, SM 35%), in 16-bit storage the FMA and shared-memory pipes (52% and 57%).  Two
 // blocks per SM (three in 16-bit storage) of 2^13 elements rather than one of
 // 2^14: three stages in one block leave FP32 pipe and shared memory idle in
 // turn (0.43-0.48 ms).
@@ -403,8 +405,9 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     if (RAG && a.late) tile_grid_wait();
 }
 
-// Bound like the strided tiles: complex64 by the memory system (0.35-0.36 ms
-// per 2^27 elements), 16-bit storage by the SM (0.19-0.21).
+// Bound like the strided tiles (0.35-0.36 ms per 2^27 elements in complex64,
+// 0.19-0.21 in 16-bit storage); whole transforms of 32 MiB in L2 by the latency of
+// their copies (long-scoreboard stalls 3.7 cycles per instruction).
 template <class G, class S, bool RAG = false>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     tile_outer_kernel(const S *__restrict__ in, S *__restrict__ out, TileArgs a) {
@@ -526,10 +529,11 @@ __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
 // of the row) beside the last axis: tile (o, y0, j) takes rows y1 Y0 + y0
 // (Y0 = n/2^RB, j: which row of the axis' stride), and frequency k1 leaves,
 // times w_n^(y0 k1), at R y0 + k1.  What is left of the axis is a strided
-// superstep of Y0 points at R times the stride.  Bound by the SM (three stages
-// over 13 bits: complex64 0.36-0.37 ms per 2^27 elements, 0.85 of the copy
-// rate; 16-bit storage 0.285-0.295); with 4096-point rows and a radix of 4,
-// tiles of 2^14 elements: 0.485 and 0.37.
+// superstep of Y0 points at R times the stride.  Bound by the latency of
+// three stages over 13 bits (complex64 0.36-0.37 ms per 2^27 elements, 0.85 of the
+// copy rate; 16-bit storage 0.285-0.295; DRAM 67%, shared memory 51%, FMA 40% busy); with
+// 4096-point rows and a radix of 4, tiles of 2^14 elements, one block per SM: 0.485
+// and 0.37 (DRAM 43%).
 template <class G, class S>
 __global__ void __launch_bounds__(1 << (G::TB - 6), TileFusedSmem<G, S>::CTAS)
     tile_wide_kernel(const S *__restrict__ in, S *__restrict__ out, TileArgs a) {
