@@ -481,9 +481,14 @@ const float2 *Plan::remember(Map &map, const Key &key, const std::vector<float2>
     if (d) map[key] = d;
     return d;
 }
+// The angles met since the last flush_tables() (null without memory: they are evaluated anew).
+RootMemo *Plan::memo() {
+    if (!roots) roots.reset(new (std::nothrow) RootMemo());
+    return roots.get();
+}
 // Copy the tables placed since the last call to the device.
 int Plan::flush_tables() {
-    roots = RootMemo();
+    roots.reset();
     for (auto &b : table_blocks) {
         if (b.pending.empty()) continue;
         const int rc = upload(b.device + b.used - b.pending.size(), b.pending.data(), b.pending.size());
@@ -510,8 +515,8 @@ const float2 *Plan::fourstep_table(int64_t L, int shift) {
     if (it != fs_tables.end()) return it->second;
     const int64_t nh = L >> shift, nl = (int64_t)1 << shift;
     std::vector<float2> h((size_t)(nh + nl));
-    for (int64_t i = 0; i < nh; ++i) h[(size_t)i] = host_root(i << shift, L, &roots);
-    for (int64_t j = 0; j < nl; ++j) h[(size_t)(nh + j)] = host_root(j, L, &roots);
+    for (int64_t i = 0; i < nh; ++i) h[(size_t)i] = host_root(i << shift, L, memo());
+    for (int64_t j = 0; j < nl; ++j) h[(size_t)(nh + j)] = host_root(j, L, memo());
     return remember(fs_tables, L, h);
 }
 
@@ -529,8 +534,8 @@ const float2 *Plan::fourstep_tile_table(int64_t L, int N) {
     const int Ns = tile_table_E(N), shift = (ilog2(L) + 1) / 2;
     const int64_t low = (int64_t)1 << shift;
     std::vector<std::complex<double>> hi((size_t)(L >> shift)), lo((size_t)low);
-    for (size_t i = 0; i < hi.size(); ++i) hi[i] = host_root_d((int64_t)i << shift, L, &roots);
-    for (size_t i = 0; i < lo.size(); ++i) lo[i] = host_root_d((int64_t)i, L, &roots);
+    for (size_t i = 0; i < hi.size(); ++i) hi[i] = host_root_d((int64_t)i << shift, L, memo());
+    for (size_t i = 0; i < lo.size(); ++i) lo[i] = host_root_d((int64_t)i, L, memo());
     std::vector<float2> h;
     h.reserve((size_t)(n1 * (Ns + N / Ns)));
     auto rows = [&](int count, int64_t step) {  // w_L^(step q j), j < count
@@ -555,7 +560,7 @@ const float2 *Plan::table(int N, int E) {
     auto key = std::make_pair(N, E);
     auto it = tables.find(key);
     if (it != tables.end()) return it->second;
-    return remember(tables, key, stage_table(N, E, &roots));
+    return remember(tables, key, stage_table(N, E, N > E ? memo() : nullptr));
 }
 
 // Twiddles of a two-stage pencil, radix R0 then N/R0: w_N^(r k) at
@@ -568,7 +573,7 @@ const float2 *Plan::table2(int N, int R0) {
     std::vector<float2> h;
     h.reserve((size_t)N);
     for (int r = 1; r < N / R0; ++r)
-        for (int k = 0; k < R0; ++k) h.push_back(host_root((int64_t)r * k, N, &roots));
+        for (int k = 0; k < R0; ++k) h.push_back(host_root((int64_t)r * k, N, memo()));
     h.push_back(make_float2(0.f, 0.f));
     return remember(tables, key, h);
 }
@@ -583,7 +588,7 @@ const float2 *Plan::class_table(int n, int classes) {
     std::vector<float2> h;
     h.reserve((size_t)n);
     for (int y = 1; y < classes; ++y)
-        for (int k = 0; k < n / classes; ++k) h.push_back(host_root((int64_t)y * k, n, &roots));
+        for (int k = 0; k < n / classes; ++k) h.push_back(host_root((int64_t)y * k, n, memo()));
     h.push_back(make_float2(0.f, 0.f));
     return remember(tables, key, h);
 }
@@ -600,7 +605,7 @@ const float2 *Plan::wide_table(int zb, int rb) {
     int64_t ns = (int64_t)1 << (5 - rb);
     for (int R : {32, (1 << zb) / (32 << (5 - rb))}) {
         for (int r = 1; r < R; ++r)
-            for (int64_t k = 0; k < ns; ++k) h.push_back(host_root(r * k, ns * R, &roots));
+            for (int64_t k = 0; k < ns; ++k) h.push_back(host_root(r * k, ns * R, memo()));
         ns *= R;
     }
     return remember(tables, key, h);
